@@ -936,62 +936,132 @@ __device__ __forceinline__ void init_ninf_tile(uint4 *tile) {
     __syncthreads();
 }
 
-// Writes one 1024-token segment of a logits row (by one warp; lane l holds
-// mask word l of the segment). A segment without an allowed token is one TMA
-// bulk copy of the -inf tile; otherwise the lanes write 16-byte chunks,
-// reading the logits only in chunks that hold an allowed token. Stores use an
-// L2 evict-first policy: the logits stream must not flush the trie tables.
 template <int kElt>
-__device__ __forceinline__ void write_segment(uint4 *__restrict__ row, int64_t c0, int64_t row_chunks,
-                                              uint32_t word, int lane, const uint4 *tile) {
+__device__ __forceinline__ void store_ninf(char *logit) {
+    if (kElt == 4) *reinterpret_cast<uint32_t *>(logit) = 0xFF800000u;
+    else *reinterpret_cast<uint16_t *>(logit) = 0xFF80u;
+}
+
+// One row of logits as the apply kernels cut it: `head` tokens before the
+// row's first 16-byte boundary (0 where V and the base are multiples of 16
+// bytes), `chunks` whole 16-byte chunks from `body`, and `tail` tokens, fewer
+// than a chunk's, after them. Segment g of the row is the 1,024 tokens from head +
+// 1024 g, so that every full segment is written by aligned 16-byte stores and
+// bulk copies whatever V is; the head goes with segment 0, the tokens after
+// the last chunk with the segment that they fall into.
+template <int kElt>
+struct RowCut {
+    char *body;
+    int32_t head;
+    int32_t chunks;
+    int32_t tail;
+
+    __device__ __forceinline__ RowCut(void *logits, int64_t b, int32_t V) {
+        char *row = static_cast<char *>(logits) + b * V * kElt;
+        head = int32_t((16u - (uint32_t(reinterpret_cast<uintptr_t>(row)) & 15u)) & 15u) / kElt;
+        head = head < V ? head : V;
+        body = row + head * kElt;
+        chunks = (V - head) / (16 / kElt);
+        tail = V - head - chunks * (16 / kElt);
+    }
+};
+
+// Writes segment seg of a cut row (by one warp): lane l holds the bits of the
+// tokens head + 1024 seg + 32 l .. + 31, head_bits (segment 0) those of the
+// tokens before the first boundary. A segment without an allowed token is one
+// TMA bulk copy of the -inf tile; otherwise the lanes write 16-byte chunks,
+// and around an allowed token only the logits beside it, so that no logit is
+// ever read: a merge of the chunk would wait for DRAM once per chunk of a lane
+// (). Whole chunks and segments are stored evict-first: the logits
+// stream must not flush the trie tables.
+template <int kElt>
+__device__ __forceinline__ void write_segment(const RowCut<kElt> &row, int32_t seg, uint32_t word,
+                                              uint32_t head_bits, int lane, const uint4 *tile) {
     constexpr int kPer = 16 / kElt;            // tokens per 16-byte chunk
     constexpr int kChunks = 1024 / kPer / 32;  // chunks per lane per segment
     constexpr int kSegChunks = 1024 / kPer;
+    const int32_t c0 = seg * kSegChunks;
+    uint4 *body = reinterpret_cast<uint4 *>(row.body);
+    if (seg == 0 && lane < row.head && !((head_bits >> lane) & 1u))
+        store_ninf<kElt>(row.body - (row.head - lane) * kElt);
+    const int32_t left = row.chunks - c0;  // whole chunks from here on
+    if (left >= 0 && left < kSegChunks && row.tail) {
+        const int32_t i = left * kPer + (lane & (kPer - 1));  // within the segment
+        const uint32_t w = __shfl_sync(0xffffffffu, word, i >> 5);
+        if (lane < row.tail && !((w >> (i & 31)) & 1u))
+            store_ninf<kElt>(row.body + (int64_t(row.chunks) * kPer + lane) * kElt);
+    }
+    if (left <= 0) return;
     if (!__any_sync(0xffffffffu, word != 0u)) {
         if (lane == 0) {
-            const int64_t nch = (row_chunks - c0 < kSegChunks) ? row_chunks - c0 : kSegChunks;
+            const int32_t nch = left < kSegChunks ? left : kSegChunks;
             const uint32_t ts = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
             uint64_t policy;
             asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;"
-                         :: "l"(row + c0), "r"(ts), "r"(uint32_t(nch * 16)), "l"(policy) : "memory");
+                         :: "l"(body + c0), "r"(ts), "r"(uint32_t(nch * 16)), "l"(policy) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // tile read before exit
         }
         return;
     }
-    const uint4 ninf = ninf16<kElt>();
+    uint32_t bits[kChunks];
+    uint4 x[kChunks];
 #pragma unroll
     for (int j = 0; j < kChunks; j++) {
         const int q = j * 32 + lane;  // chunk within the segment
         const uint32_t wv = __shfl_sync(0xffffffffu, word, (q * kPer) >> 5);
-        const uint32_t bits = (wv >> ((q * kPer) & 31)) & ((1u << kPer) - 1u);
-        const int64_t chunk = c0 + q;
-        if (chunk >= row_chunks) continue;
-        if (bits == 0u) {
-            __stcs(row + chunk, ninf);
-        } else {
-            const uint4 x = row[chunk];
-            uint32_t e[4] = {x.x, x.y, x.z, x.w};
+        bits[j] = (wv >> ((q * kPer) & 31)) & ((1u << kPer) - 1u);
+        x[j] = ninf16<kElt>();
+        if (q < left && bits[j]) x[j] = body[c0 + q];
+    }
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                if (kElt == 4) {
-                    if (!((bits >> i) & 1u)) e[i] = 0xFF800000u;
-                } else {
-                    if (!((bits >> (2 * i)) & 1u)) e[i] = (e[i] & 0xFFFF0000u) | 0xFF80u;
-                    if (!((bits >> (2 * i + 1)) & 1u)) e[i] = (e[i] & 0x0000FFFFu) | 0xFF800000u;
-                }
+    for (int j = 0; j < kChunks; j++) {
+        const int q = j * 32 + lane;
+        if (q >= left) continue;
+        uint32_t e[4] = {x[j].x, x[j].y, x[j].z, x[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            if (kElt == 4) {
+                if (!((bits[j] >> i) & 1u)) e[i] = 0xFF800000u;
+            } else {
+                if (!((bits[j] >> (2 * i)) & 1u)) e[i] = (e[i] & 0xFFFF0000u) | 0xFF80u;
+                if (!((bits[j] >> (2 * i + 1)) & 1u)) e[i] = (e[i] & 0x0000FFFFu) | 0xFF800000u;
             }
-            __stcs(row + chunk, make_uint4(e[0], e[1], e[2], e[3]));
         }
+        __stcs(body + c0 + q, make_uint4(e[0], e[1], e[2], e[3]));
     }
 }
 
-// kElt = 2 (bf16) or 4 (fp32). Requires V % (16 / kElt) == 0 and a 16-byte
-// aligned logits base, so that every row starts on a 16-byte boundary.
-// One warp per 1024-token segment of a row (one mask word per lane).
+// Masks segment seg of a cut row (by one warp) from the dense mask's row of
+// state s. The segment starts `head` < 8 tokens into a mask word, so a lane's bits
+// are its word shifted down and filled up from the next lane's; the last
+// lane's neighbour is the first word of the next segment.
 template <int kElt>
-__global__ void __launch_bounds__(kApplyThreads) k_apply_vec(uint4 *__restrict__ logits,
+__device__ __forceinline__ void mask_segment(const RowCut<kElt> &row, int32_t V, const uint32_t *__restrict__ mask,
+                                             const SegRef &sg, uint32_t ep, int32_t s, int32_t n_nodes, int64_t W,
+                                             int32_t seg, int lane, const uint4 *tile) {
+    const int64_t w0 = int64_t(seg) * 32;
+    uint32_t word = seg_row_word(mask, sg, ep, s, n_nodes, W, seg, w0 + lane, V - 1);
+    uint32_t head_bits = 0u;
+    if (row.head) {  // uniform
+        head_bits = __shfl_sync(0xffffffffu, word, 0);
+        uint32_t next = 0u;
+        if (lane == 31 && w0 + 32 < W) next = seg_row_word(mask, sg, ep, s, n_nodes, W, seg + 1, w0 + 32, V - 1);
+        const uint32_t above = __shfl_down_sync(0xffffffffu, word, 1);
+        next = lane == 31 ? next : above;
+        word = __funnelshift_r(word, next, uint32_t(row.head));
+    }
+    write_segment<kElt>(row, seg, word, head_bits, lane, tile);
+}
+
+// kElt = 2 (bf16) or 4 (fp32), logits aligned to their elements. One warp per
+// 1024-token segment of a row (one mask word per lane). Any V: a row that
+// does not start on a 16-byte boundary is cut there (RowCut). HBM-write bound:
+// B = 64, V = 128,011, bf16 3.7 us for rows of {EOS} (3.6 us at V = 128,000);
+// with one thread and one 2-byte store per logit it took 17.7 us.
+template <int kElt>
+__global__ void __launch_bounds__(kApplyThreads) k_apply_vec(void *__restrict__ logits,
                                                              const uint32_t *__restrict__ mask,
                                                              const int32_t *__restrict__ states, int32_t B,
                                                              int32_t V, int64_t W, int32_t n_nodes,
@@ -1000,16 +1070,14 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_vec(uint4 *__restrict__
     __shared__ __align__(128) uint4 tile[kSegChunks];
     init_ninf_tile<kElt>(tile);
     pdl_launch_dependents();
-    pdl_wait();  // logits and states come from earlier kernels
     const int lane = threadIdx.x & 31;
-    const int32_t item = int32_t(blockIdx.x) * (kApplyThreads / 32) + (threadIdx.x >> 5);
-    if (item >= B * segs) return;  // uniform per warp
-    const int32_t b = item / segs, seg = item - b * segs;
-    const uint32_t word = seg_row_word(mask, sg, seg_epoch_now(sg), __ldg(states + b), n_nodes, W, seg,
-                                       int64_t(seg) * 32 + lane, V - 1);
-    const int64_t row_chunks = int64_t(V) / (16 / kElt);
-    write_segment<kElt>(logits + int64_t(b) * row_chunks, int64_t(seg) * kSegChunks, row_chunks, word, lane,
-                        tile);
+    const int64_t item = int64_t(blockIdx.x) * (kApplyThreads / 32) + (threadIdx.x >> 5);
+    const int32_t b = item <= INT32_MAX ? int32_t(item) / segs : int32_t(item / segs);
+    const int32_t seg = int32_t(item - int64_t(b) * segs);
+    const RowCut<kElt> row(logits, b, V);
+    pdl_wait();  // logits and states come from earlier kernels
+    if (item >= int64_t(B) * segs) return;  // uniform per warp
+    mask_segment<kElt>(row, V, mask, sg, seg_epoch_now(sg), __ldg(states + b), n_nodes, W, seg, lane, tile);
 }
 
 // Advance, then apply, in one launch (one decode step once the sampler has
@@ -1020,7 +1088,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_vec(uint4 *__restrict__
 // (shared memory), and the CTA of part 0 stores it and counts a move into
 // DEAD.
 template <int kElt>
-__global__ void __launch_bounds__(kApplyThreads) k_advance_apply_vec(AdvanceArgs aa, uint4 *__restrict__ logits,
+__global__ void __launch_bounds__(kApplyThreads) k_advance_apply_vec(AdvanceArgs aa, void *__restrict__ logits,
                                                                      const uint32_t *__restrict__ mask,
                                                                      const int32_t *__restrict__ states_in,
                                                                      const int32_t *__restrict__ tokens,
@@ -1034,6 +1102,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_advance_apply_vec(AdvanceArgs
     __shared__ uint32_t epoch;
     pdl_launch_dependents();
     const int32_t b = int32_t(blockIdx.x) / parts, part = int32_t(blockIdx.x) - b * parts;
+    const RowCut<kElt> row(logits, b, aa.V);
     for (int i = threadIdx.x; i < kSegChunks; i += blockDim.x) tile[i] = ninf16<kElt>();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // tile visible to the bulk copies
     if (threadIdx.x == 0) {
@@ -1052,11 +1121,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_advance_apply_vec(AdvanceArgs
     const int lane = threadIdx.x & 31;
     const int32_t seg = part * (kApplyThreads / 32) + int32_t(threadIdx.x >> 5);
     if (seg >= segs) return;  // uniform per warp
-    const uint32_t word = seg_row_word(mask, sg, epoch, next_state, aa.n_nodes, W, seg,
-                                       int64_t(seg) * 32 + lane, aa.V - 1);
-    const int64_t row_chunks = int64_t(aa.V) / (16 / kElt);
-    write_segment<kElt>(logits + int64_t(b) * row_chunks, int64_t(seg) * kSegChunks, row_chunks, word, lane,
-                        tile);
+    mask_segment<kElt>(row, aa.V, mask, sg, epoch, next_state, aa.n_nodes, W, seg, lane, tile);
 }
 
 // ---------------------------------------------------------------- valid lists
@@ -1315,12 +1380,12 @@ __global__ void __launch_bounds__(kWalkThreads) k_list_walk(WalkArgs a) {
     for (int32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < a.n_nodes; m += stride) walk_node(a, root, m, tok);
 }
 // Apply from the lists: CTA (row b, part p) covers 8 segments (8,192 tokens).
-// It rebuilds their 256 mask words in shared memory from the row's list and
-// writes them like k_apply_vec (kVec) or one logit per thread (any V and
-// alignment). With kAdvance the row's state is first moved by its token
+// It rebuilds their 256 mask words (counted from the row's first 16-byte
+// boundary) and the head's bits in shared memory from the row's list and
+// writes them like k_apply_vec. With kAdvance the row's state is first moved by its token
 // (thread 0; the CTA of part 0 stores it and counts a move into DEAD): the
 // advance of one decode step and the apply of the next in one launch.
-template <int kElt, bool kVec, bool kAdvance>
+template <int kElt, bool kAdvance>
 __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict__ logits,
                                                                const int64_t *__restrict__ off,
                                                                const int32_t *__restrict__ toks, AdvanceArgs aa,
@@ -1332,16 +1397,19 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict_
                                                                const int32_t *__restrict__ ends) {
     constexpr int kSegChunks = 1024 / (16 / kElt);
     constexpr int kWords = 8 * 32;
-    __shared__ __align__(128) uint4 tile[kVec ? kSegChunks : 1];
-    __shared__ uint32_t words[kWords];
+    __shared__ __align__(128) uint4 tile[kSegChunks];
+    __shared__ uint32_t words[kWords], head_bits;
     __shared__ int32_t state, moved;
     for (int i = threadIdx.x; i < kWords; i += kApplyThreads) words[i] = 0u;
-    if (threadIdx.x == 0) moved = kDead;
-    if (kVec) init_ninf_tile<kElt>(tile);
-    else __syncthreads();
+    if (threadIdx.x == 0) {
+        moved = kDead;
+        head_bits = 0u;
+    }
+    init_ninf_tile<kElt>(tile);
     pdl_launch_dependents();
-    pdl_wait();  // logits, states and tokens come from earlier kernels
     const int32_t b = int32_t(blockIdx.x) / parts, part = int32_t(blockIdx.x) - b * parts;
+    const RowCut<kElt> row(logits, b, V);
+    pdl_wait();  // logits, states and tokens come from earlier kernels
     const int32_t s0 = __ldg(states + b);
     if (kAdvance) {
         // from a node, the move is the entry of the token in the node's list
@@ -1371,55 +1439,21 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict_
     }
     __syncthreads();
     const int32_t s = state;
-    const int32_t t0 = part * 8192, eos = V - 1;
+    const int32_t t0 = part * 8192 + row.head, eos = V - 1;
+    auto set_bit = [&](int32_t v) {
+        const int32_t t = v - t0;
+        if (t >= 0 && t < 8192) atomicOr(words + (t >> 5), 1u << (t & 31));
+        else if (v < row.head) atomicOr(&head_bits, 1u << v);
+    };
     if (s >= 0 && s < n_nodes) {
         const int64_t lo = __ldg(off + s), hi = __ldg(off + s + 1);
-        for (int64_t i = lo + threadIdx.x; i < hi; i += kApplyThreads) {
-            const int32_t t = __ldg(toks + i) - t0;
-            if (t >= 0 && t < 8192) atomicOr(words + (t >> 5), 1u << (t & 31));
-        }
-    } else if (threadIdx.x == 0 && eos - t0 >= 0 && eos - t0 < 8192) {
-        words[(eos - t0) >> 5] = 1u << ((eos - t0) & 31);  // FINISHED, DEAD, not a node: {EOS}
+        for (int64_t i = lo + threadIdx.x; i < hi; i += kApplyThreads) set_bit(__ldg(toks + i));
+    } else if (threadIdx.x == 0) {
+        set_bit(eos);  // FINISHED, DEAD, not a node: {EOS}
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (kVec) {
-        const int64_t row_chunks = int64_t(V) / (16 / kElt);
-        const int64_t c0 = (int64_t(part) * 8 + wid) * kSegChunks;
-        if (c0 >= row_chunks) return;
-        write_segment<kElt>(static_cast<uint4 *>(logits) + int64_t(b) * row_chunks, c0, row_chunks,
-                            words[wid * 32 + lane], lane, tile);
-    } else {
-        for (int32_t j = threadIdx.x; j < 8192; j += kApplyThreads) {
-            const int32_t v = t0 + j;
-            if (v >= V) break;
-            if ((words[j >> 5] >> (j & 31)) & 1u) continue;
-            const int64_t idx = int64_t(b) * V + v;
-            if (kElt == 4) static_cast<uint32_t *>(logits)[idx] = 0xFF800000u;
-            else static_cast<uint16_t *>(logits)[idx] = 0xFF80u;
-        }
-    }
-}
-
-// Any V and alignment: one thread per logit.
-template <int kElt>
-__global__ void __launch_bounds__(kApplyThreads) k_apply_scalar(void *__restrict__ logits,
-                                                                const uint32_t *__restrict__ mask,
-                                                                const int32_t *__restrict__ states,
-                                                                int32_t B, int32_t V, int64_t W,
-                                                                int32_t n_nodes) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int64_t total = int64_t(B) * V;
-    const int32_t eos = V - 1;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t b = int32_t(i / V), v = int32_t(i % V);
-        const uint32_t word = row_word(mask, __ldg(states + b), n_nodes, W, v >> 5, eos);
-        if ((word >> (v & 31)) & 1u) continue;
-        if (kElt == 4) static_cast<uint32_t *>(logits)[i] = 0xFF800000u;
-        else static_cast<uint16_t *>(logits)[i] = 0xFF80u;
-    }
+    write_segment<kElt>(row, part * 8 + wid, words[wid * 32 + lane], head_bits, lane, tile);
 }
 
 // ------------------------------------------------------------ lazy rows
@@ -1980,50 +2014,37 @@ cudaError_t launch_advance(const DevTrie &t, int32_t n_nodes, const DevVocab &v,
 cudaError_t launch_advance_apply(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bool use_trans,
                                  const int32_t *states_in, const int32_t *tokens, int32_t *states_out,
                                  int32_t *err, void *logits, int dtype, const uint32_t *mask, int32_t B,
-                                 int num_sms, cudaStream_t st, const SegRef &seg) {
+                                 cudaStream_t st, const SegRef &seg) {
     const int32_t V = v.V;
     const int64_t W = (int64_t(V) + 31) / 32;
     const int elt = dtype == 0 ? 4 : 2;
     const int32_t segs = int32_t((W + 31) / 32);
-    const bool vec = (reinterpret_cast<uintptr_t>(logits) & 15u) == 0 && (int64_t(V) * elt) % 16 == 0 &&
-                     int64_t(B) * segs < int64_t(INT32_MAX);
-    if (!vec) {  // any V and alignment: the two kernels one after the other
-        cudaError_t e = launch_advance(t, n_nodes, v, states_in, states_out, tokens, B, err, use_trans, st);
-        if (e != cudaSuccess) return e;
-        return launch_apply(logits, dtype, mask, states_out, B, V, n_nodes, num_sms, st, seg);
-    }
-    const AdvanceArgs aa = advance_args(t, n_nodes, v, use_trans);
     const int32_t parts = (segs + kApplyThreads / 32 - 1) / (kApplyThreads / 32);
     const int64_t grid = int64_t(B) * parts;
-    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    if (grid > INT32_MAX) {  // more CTAs than a grid holds: the two kernels one after the other
+        cudaError_t e = launch_advance(t, n_nodes, v, states_in, states_out, tokens, B, err, use_trans, st);
+        if (e != cudaSuccess) return e;
+        return launch_apply(logits, dtype, mask, states_out, B, V, n_nodes, st, seg);
+    }
+    const AdvanceArgs aa = advance_args(t, n_nodes, v, use_trans);
     if (elt == 2)
-        return launch_pdl(k_advance_apply_vec<2>, grid, kApplyThreads, st, aa, static_cast<uint4 *>(logits), mask,
-                          states_in, tokens, states_out, err, B, W, segs, parts, seg);
-    return launch_pdl(k_advance_apply_vec<4>, grid, kApplyThreads, st, aa, static_cast<uint4 *>(logits), mask,
-                      states_in, tokens, states_out, err, B, W, segs, parts, seg);
+        return launch_pdl(k_advance_apply_vec<2>, grid, kApplyThreads, st, aa, logits, mask, states_in, tokens,
+                          states_out, err, B, W, segs, parts, seg);
+    return launch_pdl(k_advance_apply_vec<4>, grid, kApplyThreads, st, aa, logits, mask, states_in, tokens,
+                      states_out, err, B, W, segs, parts, seg);
 }
 
 cudaError_t launch_apply(void *logits, int dtype, const uint32_t *mask, const int32_t *states,
-                         int32_t B, int32_t V, int32_t n_nodes, int num_sms, cudaStream_t st,
-                         const SegRef &seg) {
+                         int32_t B, int32_t V, int32_t n_nodes, cudaStream_t st, const SegRef &seg) {
     const int64_t W = (int64_t(V) + 31) / 32;
-    const int elt = dtype == 0 ? 4 : 2;
     const int32_t segs = int32_t((W + 31) / 32);
-    const bool vec = (reinterpret_cast<uintptr_t>(logits) & 15u) == 0 && (int64_t(V) * elt) % 16 == 0 &&
-                     int64_t(B) * segs < int64_t(INT32_MAX);
-    if (vec) {
-        const int64_t items = int64_t(B) * segs;
-        const int grid = grid_for(items, kApplyThreads / 32, INT32_MAX);
-        if (elt == 2)
-            return launch_pdl(k_apply_vec<2>, grid, kApplyThreads, st, static_cast<uint4 *>(logits), mask,
-                              states, B, V, W, n_nodes, segs, seg);
-        return launch_pdl(k_apply_vec<4>, grid, kApplyThreads, st, static_cast<uint4 *>(logits), mask, states,
-                          B, V, W, n_nodes, segs, seg);
-    }
-    const int grid = grid_for(int64_t(B) * V, kApplyThreads, int64_t(num_sms) * 16);
-    if (elt == 2)
-        return launch_pdl(k_apply_scalar<2>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes);
-    return launch_pdl(k_apply_scalar<4>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes);
+    // more CTAs than a grid holds would mean more logits than any device does
+    const int64_t grid = (int64_t(B) * segs + kApplyThreads / 32 - 1) / (kApplyThreads / 32);
+    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    if (dtype == 0)
+        return launch_pdl(k_apply_vec<4>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes, segs,
+                          seg);
+    return launch_pdl(k_apply_vec<2>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes, segs, seg);
 }
 
 namespace {
@@ -2138,34 +2159,16 @@ namespace {
 cudaError_t launch_lists(void *logits, int dtype, const DevLists &L, const AdvanceArgs *aa,
                          const int32_t *states, const int32_t *tokens, int32_t *states_out, int32_t *err,
                          int32_t B, int32_t V, int32_t n_nodes, cudaStream_t st) {
-    const int elt = dtype == 0 ? 4 : 2;
     const int32_t parts = int32_t((int64_t(V) + 8191) / 8192);
-    const bool vec = (reinterpret_cast<uintptr_t>(logits) & 15u) == 0 && (int64_t(V) * elt) % 16 == 0;
     const int64_t grid = int64_t(B) * parts;
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
     const int32_t *tk = L.toks;
     const int64_t *of = L.off;
     const AdvanceArgs a = aa ? *aa : AdvanceArgs{};
-    if (aa) {
-        if (vec)
-            return elt == 2 ? launch_pdl(k_apply_lists<2, true, true>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                         states, tokens, states_out, err, B, V, n_nodes, parts, L.ends)
-                            : launch_pdl(k_apply_lists<4, true, true>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                         states, tokens, states_out, err, B, V, n_nodes, parts, L.ends);
-        return elt == 2 ? launch_pdl(k_apply_lists<2, false, true>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                     states, tokens, states_out, err, B, V, n_nodes, parts, L.ends)
-                        : launch_pdl(k_apply_lists<4, false, true>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                     states, tokens, states_out, err, B, V, n_nodes, parts, L.ends);
-    }
-    if (vec)
-        return elt == 2 ? launch_pdl(k_apply_lists<2, true, false>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                     states, tokens, states_out, err, B, V, n_nodes, parts, L.ends)
-                        : launch_pdl(k_apply_lists<4, true, false>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                     states, tokens, states_out, err, B, V, n_nodes, parts, L.ends);
-    return elt == 2 ? launch_pdl(k_apply_lists<2, false, false>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                 states, tokens, states_out, err, B, V, n_nodes, parts, L.ends)
-                    : launch_pdl(k_apply_lists<4, false, false>, int(grid), kApplyThreads, st, logits, of, tk, a,
-                                 states, tokens, states_out, err, B, V, n_nodes, parts, L.ends);
+    auto *kernel = dtype == 0 ? (aa ? k_apply_lists<4, true> : k_apply_lists<4, false>)
+                              : (aa ? k_apply_lists<2, true> : k_apply_lists<2, false>);
+    return launch_pdl(kernel, grid, kApplyThreads, st, logits, of, tk, a, states, tokens, states_out, err, B, V,
+                      n_nodes, parts, L.ends);
 }
 
 }  // namespace
@@ -2246,7 +2249,7 @@ cudaError_t launch_lazy(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bo
     e = launch_pdl_smem(k_lazy_rows, rows_grid, kLazyRowThreads, size_t(L.W) * sizeof(uint32_t), st, la, pa);
     if (e != cudaSuccess) return e;
     const int32_t n_rows = L.C + L.max_batch;
-    if (logits) return launch_apply(logits, dtype, L.rows, L.slot_of, B, L.V, n_rows, num_sms, st);
+    if (logits) return launch_apply(logits, dtype, L.rows, L.slot_of, B, L.V, n_rows, st);
     const int grid = grid_for(int64_t(B) * L.W, kApplyThreads, int64_t(num_sms) * 8);
     return launch_pdl(k_lazy_gather, grid, kApplyThreads, st, static_cast<const uint32_t *>(L.rows),
                       static_cast<const int32_t *>(L.slot_of), B, L.W, n_rows, L.V - 1, rows_out);
