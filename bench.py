@@ -898,10 +898,10 @@ def run_dynamic(dev, stream, steps: int = 32, reps: int = 5, rank: int = 0, worl
     out["list_entries"] = n_valid
     out["list_bytes"] = n_valid * 4 + (N + 1) * 8
     # the list compile's algorithmic traffic: the entries and offsets written
-    # plus the per-node tables the walks read (window 16 B, anc 64 B, depth,
-    # terminal: 82 B per node, read by both walks)
+    # plus the trie's arrays the walks read (parent 4 B, label, terminal: 6 B
+    # per node, read by both walks)
     peak, peak_kind = peaks()
-    list_bytes = out["list_bytes"] + 2 * 82 * N
+    list_bytes = out["list_bytes"] + 2 * 6 * N
     out["roofline_lists"] = {"bound": "hbm", "achieved": list_bytes / (min(lt) * 1e-3) / 1e9, "peak": peak,
                              "unit": "GB/s", "frac": list_bytes / (min(lt) * 1e-3) / 1e9 / peak,
                              "bytes_per_launch": list_bytes, "peak_kind": peak_kind,

@@ -48,8 +48,9 @@
  * passes (mask, states, tokens, logits, error counter). The mask passed to
  * trie_compile_masks must stay allocated and unchanged while the handle is
  * used by trie_apply_mask (the handle keeps a non-owning pointer to it).
- * A handle's device memory (trie arrays and per-node tables, 123 B per
- * node, plus a transition table of at least 128 B per node for a single trie;
+ * A handle's device memory (trie arrays, 42 B per node; the dense compile's
+ * and lazy rows' tables, 81 B per node, allocated by a forest's first such
+ * call; a transition table of at least 128 B per node for a single trie;
  * the dense compile's hit buffer, 129 B per node, allocated by the
  * handle's first trie_compile_masks; valid lists; lazy rows) and the
  * scratch of trie_build_many_device come from a memory pool per device that
@@ -124,8 +125,8 @@ int trie_build_many(const uint8_t *bytes, const int64_t *offsets, const int32_t 
  * environment forces the copies). The offsets are checked on the device.
  * Returns once the node count and the roots are known on the host (read back
  * after the level insertion; the caller's arrays have been read by then):
- * the last kernels (the breadth-first layout, child links and per-node
- * tables) are still queued on `stream`, so use the handle on `stream` or
+ * the last kernels (the breadth-first layout and the child links) are still
+ * queued on `stream`, so use the handle on `stream` or
  * after synchronising it (calls that copy arrays back synchronise the device
  * first); an error in those kernels surfaces on a later call. Such a
  * forest has no transition table: trie_advance and the fused calls walk the

@@ -187,21 +187,33 @@ int get_vocab(const uint8_t *vb, const int64_t *vo, int32_t V, int dev,
 // Uploads the trie on first use, ordered on `stream` (the copies read the
 // handle's own host arrays, which outlive them); the handle is bound to that
 // device.
+// Places the per-node compile tables (window, depth16, anc) in a layout.
+struct TableLayout {
+    size_t win, d16, anc;
+    TableLayout(Layout &L, size_t n)
+        : win(L.add(sizeof(uint64_t) * 2 * n)), d16(L.add(n)), anc(L.add(sizeof(int32_t) * 16 * n)) {}
+    void place(tmk::DevTrie *t, char *b) const {
+        t->window = reinterpret_cast<ulonglong2 *>(b + win);
+        t->depth16 = reinterpret_cast<uint8_t *>(b + d16);
+        t->anc = reinterpret_cast<int4 *>(b + anc);
+    }
+};
+
 // Device arrays of a trie of n nodes (one allocation); nothing is uploaded.
-// with_trans: also a transition table (8 or more slots per node) for the
-// compiles to record moves in.
-int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool with_trans) {
+// single: a single trie, which gets the compile tables at once and a
+// transition table (8 or more slots per node) for the compiles to record
+// moves in. A forest gets the tables on its first dense compile or lazy
+// set-up (ensure_tables): its valid lists need neither.
+int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool single) {
     Layout L;
     const size_t o_par = L.add(sizeof(int32_t) * n);
     const size_t o_lab = L.add(n);
     const size_t o_term = L.add(n);
     const size_t o_fc = L.add(sizeof(int32_t) * n);
     const size_t o_bits = L.add(sizeof(uint32_t) * 8 * n);
-    const size_t o_win = L.add(sizeof(uint64_t) * 2 * n);
-    const size_t o_d16 = L.add(n);
-    const size_t o_anc = L.add(sizeof(int32_t) * 16 * n);
-    size_t trans_slots = with_trans ? 16 : 0;  // >= 8 per node, a power of two
-    while (with_trans && trans_slots < 8 * n) trans_slots <<= 1;
+    const TableLayout tables(L, single ? n : 0);
+    size_t trans_slots = single ? 16 : 0;  // >= 8 per node, a power of two
+    while (single && trans_slots < 8 * n) trans_slots <<= 1;
     const size_t o_trans = L.add(sizeof(ulonglong2) * trans_slots);
     void *base = nullptr;
     const int rc = pool_alloc(dev, L.total, stream, &base, "the trie");
@@ -214,25 +226,45 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool wit
     h->dev.terminal = reinterpret_cast<const uint8_t *>(b + o_term);
     h->dev.first_child = reinterpret_cast<int32_t *>(b + o_fc);
     h->dev.child_bits = reinterpret_cast<uint32_t *>(b + o_bits);
-    h->dev.window = reinterpret_cast<ulonglong2 *>(b + o_win);
-    h->dev.depth16 = reinterpret_cast<uint8_t *>(b + o_d16);
-    h->dev.anc = reinterpret_cast<int4 *>(b + o_anc);
-    h->dev.trans = with_trans ? reinterpret_cast<ulonglong2 *>(b + o_trans) : nullptr;
-    h->dev.trans_mask = with_trans ? uint32_t(trans_slots - 1) : 0u;
+    if (single) tables.place(&h->dev, b);
+    h->dev.trans = single ? reinterpret_cast<ulonglong2 *>(b + o_trans) : nullptr;
+    h->dev.trans_mask = single ? uint32_t(trans_slots - 1) : 0u;
     return TRIE_OK;
 }
 
-// The child links and the compile's per-node tables, from the device's
+// The child links, and a single trie's compile tables, from the device's
 // parent / label / terminal arrays (once they are written on `stream`).
 int finish_device_trie(trie_t h, int dev, cudaStream_t stream) {
-    cudaError_t e;
-    if ((e = tmk::launch_trie_links(h->dev, h->host.n, num_sms(dev), stream)) == cudaSuccess)
-        e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
+    cudaError_t e = tmk::launch_trie_links(h->dev, h->host.n, num_sms(dev), stream);
+    if (e == cudaSuccess && h->dev.window) e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
     if (e != cudaSuccess) {
         pool_free(h->dev.base);
         h->dev = tmk::DevTrie();
         return fail_cuda(e, "building the trie's compile tables");
     }
+    return TRIE_OK;
+}
+
+// A forest's compile tables, on the first call that reads them (81 B and 16
+// dependent loads per node: 80 us and 386 MB for 4.77 M nodes that a forest
+// compiled to lists never uses). The caller must be a call that does not run
+// beside others on the handle.
+int ensure_tables(trie_t h, int dev, cudaStream_t stream) {
+    std::lock_guard<std::mutex> lk(h->mu);
+    if (h->dev.window) return TRIE_OK;
+    Layout L;
+    const TableLayout tables(L, size_t(h->host.n));
+    void *base = nullptr;
+    const int rc = pool_alloc(dev, L.total, stream, &base, "the trie's compile tables");
+    if (rc != TRIE_OK) return rc;
+    tables.place(&h->dev, static_cast<char *>(base));
+    const cudaError_t e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
+    if (e != cudaSuccess) {
+        h->dev.window = nullptr;
+        pool_free(base);
+        return fail_cuda(e, "building the trie's compile tables");
+    }
+    h->dev.tables_base = base;
     return TRIE_OK;
 }
 
@@ -573,7 +605,7 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
     }
     // no synchronisation here: the node count and roots are on the host, the
     // caller's arrays have been read, and the last kernels (breadth-first
-    // layout, child links, per-node tables) finish on `stream` while the host
+    // layout, child links) finish on `stream` while the host
     // goes on (a later call on `stream` is ordered after them)
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -685,6 +717,7 @@ static int compile_masks(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
     int rc;
     const int32_t V = voc->V;
     if ((rc = ensure_device_trie(h, dev, stream)) != TRIE_OK) return rc;
+    if ((rc = ensure_tables(h, dev, stream)) != TRIE_OK) return rc;
     if ((rc = ensure_hits(h, dev, stream)) != TRIE_OK) return rc;
     const int64_t W = (int64_t(V) + 31) / 32;
     const int32_t n = h->host.n;
@@ -1060,7 +1093,7 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
         return r;
     };
     if (by_bound && (rc = grow(bound)) != TRIE_OK) return failed(rc);
-    cudaError_t e = tmk::launch_lists_count(h->dev, n, *voc, lmax, L, sms, stream);
+    cudaError_t e = tmk::launch_lists_count(h->dev, n, *voc, L, sms, stream);
     if (e != cudaSuccess) return failed(fail_cuda(e, "valid-list count"));
     if (!by_bound) {
         int64_t total = 0;
@@ -1069,7 +1102,7 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
             return failed(fail_cuda(e, "reading the number of list entries back"));
         if ((rc = grow(total + total / 2)) != TRIE_OK) return failed(rc);
     }
-    e = tmk::launch_lists_write(h->dev, n, *voc, lmax, L, sms, stream);
+    e = tmk::launch_lists_write(h->dev, n, *voc, L, sms, stream);
     if (e == cudaSuccess) e = cudaEventRecord(L.done, stream);
     if (e != cudaSuccess) return failed(fail_cuda(e, "valid-list write"));
     std::lock_guard<std::mutex> lk(h->mu);
@@ -1191,6 +1224,7 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     if ((rc = get_vocab(vocab_bytes, vocab_offsets, V, dev, &voc)) != TRIE_OK) return rc;
     if ((rc = tmk::ensure_host_arrays(h)) != TRIE_OK) return rc;  // the pre-order tables
     if ((rc = ensure_device_trie(h, dev, 0)) != TRIE_OK) return rc;
+    if ((rc = ensure_tables(h, dev, 0)) != TRIE_OK) return rc;
     cudaError_t e = cudaDeviceSynchronize();  // earlier lazy calls may still use the old cache
     if (e != cudaSuccess) return fail_cuda(e, "synchronising before the lazy set-up");
     {  // the transition table takes the moves the lazy rows find for this vocabulary
@@ -1465,6 +1499,7 @@ int trie_destroy(trie_t h) {
             give_spare_block(h->dev.device, h->lists.base, h->lists.base_bytes, nullptr, 0);
         }
         pool_free(h->dev.hits_base);
+        pool_free(h->dev.tables_base);
         pool_free(h->dev.seg_epoch);
         pool_free(h->dev.base);
         if (h->lists.done) cudaEventDestroy(h->lists.done);
@@ -1543,6 +1578,7 @@ int trie_destroy_async(trie_t h, cudaStream_t stream) {
             }
         }
         free_on(h->dev.hits_base);
+        free_on(h->dev.tables_base);
         free_on(h->dev.seg_epoch);
         free_on(h->dev.base);
         // the event may still be pending: CUDA defers its destruction

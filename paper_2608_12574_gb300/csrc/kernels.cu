@@ -1246,13 +1246,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_rows(const int32_t *__res
 
 struct WalkArgs {
     const uint8_t *terminal;
-    const ulonglong2 *window;  // last 16 labels into each node (byte i = i levels up)
-    const uint8_t *depth16;    // min(depth, 16)
-    const int32_t *anc;        // [n * 16]: ancestors 1..16 levels up
     const int32_t *parent;
     const uint8_t *label;
     int32_t n_nodes;
-    int32_t lmax;              // min(longest token, trie depth)
     int32_t eos;
     const uint4 *edge;         // {(parent << 8 | byte) + 1, child, token or -1, 0}; key 0 = empty
     uint32_t edge_mask;        // slots - 1
@@ -1309,37 +1305,37 @@ __global__ void k_rt_insert(const int32_t *__restrict__ parent, const uint8_t *_
 // Every (row, token) entry whose path ends at node m: EOS at m if m is
 // terminal (App. G.5), then the tokens met by the walk (row = the node as
 // many levels above m as the token has bytes). root[c] = {child, token} of
-// the reversed trie's root for byte c.
+// the reversed trie's root for byte c. The climb reads each level's parent
+// and label itself, one level ahead of the edge it looks up: neighbouring
+// nodes' ancestors are neighbours, so these loads fall together and come from
+// L1 and L2, where reading each entry's row from the 64-byte ancestor rows of
+// the dense compile's tables was 305 MB of DRAM reads a walk on the 4.77 M-node
+// forest (count walk 132 us, 104 us so; write walk 177 and 143 us; and the
+// forest needs no such tables). Called by whole warps, whose lanes stay
+// together until the longest walk ends: with a return at each lane's own end
+// the lanes ran on one by one (326 and 520 us).
 template <typename Tok>
 __device__ __forceinline__ void walk_node(const WalkArgs &a, const int2 *root, int32_t m, Tok tok) {
-    if (__ldg(a.terminal + m)) tok(m, a.eos, kFinished);
-    const int32_t d16 = __ldg(a.depth16 + m);
-    const int32_t lim = a.lmax < d16 ? a.lmax : d16;
-    if (lim <= 0) return;
-    const ulonglong2 win = __ldg(a.window + m);
-    const int32_t *up = a.anc + int64_t(m) * 16;
-    const int2 r0 = root[uint32_t(win.x) & 0xFFu];
-    int32_t x = r0.x;
-    if (x < 0) return;
-    if (r0.y >= 0) tok(__ldg(up), r0.y, m);
-    for (int32_t j = 1; j < lim; j++) {
-        const uint32_t c = uint32_t((j < 8 ? win.x >> (8 * j) : win.y >> (8 * (j - 8))) & 0xFFu);
-        uint4 e;
-        if (!rt_step(a.edge, a.edge_mask, a.edge_shift, x, c, &e)) return;
-        x = int32_t(e.y);
-        if (int32_t(e.z) >= 0) tok(__ldg(up + j), int32_t(e.z), m);
+    int32_t p = -1, x = -1, t = -1;
+    uint32_t c = 0u;
+    if (m < a.n_nodes) {
+        p = __ldg(a.parent + m);
+        c = __ldg(a.label + m);
+        if (__ldg(a.terminal + m)) tok(m, a.eos, kFinished);
+        x = root[c].x;
+        t = root[c].y;
     }
-    // tokens longer than the 16-label window, in a trie deeper than 16
-    if (lim == 16 && a.lmax > 16) {
-        int32_t y = __ldg(up + 15);  // 16 levels above m: its label is the 17th
-        for (int32_t j = 16; j < a.lmax; j++) {
-            const int32_t p = __ldg(a.parent + y);
-            if (p < 0) return;
+    bool on = p >= 0 && x >= 0;
+    while (__any_sync(0xffffffffu, on)) {  // (x, t): the edge taken by the label below p
+        const int32_t row = p;
+        if (on) {
+            p = __ldg(a.parent + row);
+            c = __ldg(a.label + row);
+            if (t >= 0) tok(row, t, m);
             uint4 e;
-            if (!rt_step(a.edge, a.edge_mask, a.edge_shift, x, __ldg(a.label + y), &e)) return;
+            on = p >= 0 && rt_step(a.edge, a.edge_mask, a.edge_shift, x, c, &e);
             x = int32_t(e.y);
-            if (int32_t(e.z) >= 0) tok(p, int32_t(e.z), m);
-            y = p;
+            t = int32_t(e.z);
         }
     }
 }
@@ -1377,8 +1373,10 @@ __global__ void __launch_bounds__(kWalkThreads) k_list_walk(WalkArgs a) {
             for (int32_t u = __ldg(a.tok_next + t); u >= 0; u = __ldg(a.tok_next + u)) emit(row, u, end);
     };
     const int32_t stride = gridDim.x * blockDim.x;
-    for (int32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < a.n_nodes; m += stride) walk_node(a, root, m, tok);
+    for (int32_t m0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); m0 < a.n_nodes; m0 += stride)
+        walk_node(a, root, m0 + int32_t(threadIdx.x & 31), tok);
 }
+
 // Apply from the lists: CTA (row b, part p) covers 8 segments (8,192 tokens).
 // It rebuilds their 256 mask words (counted from the row's first 16-byte
 // boundary) and the head's bits in shared memory from the row's list and
@@ -2103,16 +2101,12 @@ cudaError_t launch_rt_build(const int32_t *parent, const uint8_t *label, const i
 
 namespace {
 
-WalkArgs walk_args(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t lmax, const DevLists &L) {
+WalkArgs walk_args(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L) {
     WalkArgs a;
     a.terminal = t.terminal;
-    a.window = t.window;
-    a.depth16 = t.depth16;
-    a.anc = reinterpret_cast<const int32_t *>(t.anc);
     a.parent = t.parent;
     a.label = t.label;
     a.n_nodes = n_nodes;
-    a.lmax = lmax;
     a.eos = v.V - 1;
     a.edge = v.rt_edge;
     a.edge_mask = v.rt_mask;
@@ -2128,9 +2122,9 @@ WalkArgs walk_args(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t
 
 }  // namespace
 
-cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t lmax,
-                               const DevLists &L, int num_sms, cudaStream_t st) {
-    const WalkArgs a = walk_args(t, n_nodes, v, lmax, L);
+cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
+                               int num_sms, cudaStream_t st) {
+    const WalkArgs a = walk_args(t, n_nodes, v, L);
     cudaError_t e = launch_mask_fill(reinterpret_cast<uint32_t *>(L.count), int64_t(n_nodes), num_sms, st);
     if (e != cudaSuccess) return e;
     const int grid = grid_for(n_nodes, kWalkThreads, int64_t(num_sms) * 8);
@@ -2147,9 +2141,9 @@ cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab
     return cudaSuccess;
 }
 
-cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t lmax,
-                               const DevLists &L, int num_sms, cudaStream_t st) {
-    const WalkArgs a = walk_args(t, n_nodes, v, lmax, L);
+cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
+                               int num_sms, cudaStream_t st) {
+    const WalkArgs a = walk_args(t, n_nodes, v, L);
     const int grid = grid_for(n_nodes, kWalkThreads, int64_t(num_sms) * 8);
     return launch_pdl(k_list_walk<true>, grid, kWalkThreads, st, a);
 }

@@ -245,10 +245,11 @@ struct DevTrie {
     const uint8_t *terminal = nullptr;
     int32_t *first_child = nullptr;      // built on the device (launch_trie_links)
     uint32_t *child_bits = nullptr;      // [n * 8], built on the device
-    // Per node, for the mask compile, built on the device from parent/label
-    // (launch_trie_tables): the labels of the last 16 edges into it (byte i =
-    // label i levels up, 0 past the root), min(depth, 16), and the ancestors
-    // 1..16 levels up (entry k = k + 1 levels up, -1 past the root).
+    // Per node, for the dense compile and the lazy rows, built on the device
+    // from parent/label (launch_trie_tables; null until a forest's first use):
+    // the labels of the last 16 edges into it (byte i = label i levels up, 0
+    // past the root), min(depth, 16), and the ancestors 1..16 levels up (entry
+    // k = k + 1 levels up, -1 past the root).
     ulonglong2 *window = nullptr;    // [n]
     uint8_t *depth16 = nullptr;      // [n]
     int4 *anc = nullptr;             // [n * 4]
@@ -263,6 +264,7 @@ struct DevTrie {
     uint32_t *seg_epoch = nullptr;          // [1] (device), the epoch of the last compile that ran
     uint32_t seg_epoch_next = 1;            // host: the epoch of the next compile (0 is never used)
     int64_t seg_cap = 0;
+    void *tables_base = nullptr;     // a forest's window, depth16 and anc (own allocation)
     void *hits_base = nullptr;       // the two arrays below (allocated by the first dense compile)
     int2 *hits = nullptr;            // compile scratch: kHitSlots (row, token) pairs per node
     uint8_t *hit_count = nullptr;    // compile scratch: hits found per node
@@ -482,10 +484,10 @@ cudaError_t launch_rt_build(const int32_t *parent, const uint8_t *label, const i
 // i) and *L.total. Write: walk again, writing every entry at the position
 // claimed from off[row + 1] into L.toks (entries past L.tok_cap are
 // dropped); afterwards L.off holds the rows' offsets.
-cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t lmax,
-                               const DevLists &L, int num_sms, cudaStream_t st);
-cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, int32_t lmax,
-                               const DevLists &L, int num_sms, cudaStream_t st);
+cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
+                               int num_sms, cudaStream_t st);
+cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
+                               int num_sms, cudaStream_t st);
 // Lazy rows: pos_of from the pre-order tables and the path hashes (once, at set-up).
 cudaError_t launch_lazy_tables(const DevTrie &t, const DevLazy &L, int32_t n_nodes, cudaStream_t st);
 // One lazy call: map the batch's states (after the advance when tokens is not

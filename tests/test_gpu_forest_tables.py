@@ -1,0 +1,44 @@
+"""A forest has no compile tables until a call reads them: lists first, then
+the dense compile or the lazy rows of the same handle, and a synchronous and
+a stream-ordered release of each."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_12574_gb300 import triemask as T
+from paper_2608_12574_gb300 import workloads as W
+from pins import random_case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("then", ["masks", "lazy"])
+@pytest.mark.parametrize("device_build", [False, True])
+@pytest.mark.parametrize("lists_first", [False, True])
+def test_tables_on_first_use(then, device_build, lists_first):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    oracle.build()
+    strings, toks = random_case(91)
+    sets = [strings, strings[:3] + [b""], [x + b"a" * 20 for x in strings]]
+    sb, so = W.pack([x for s in sets for x in s])
+    si = np.cumsum([0] + [len(s) for s in sets]).astype(np.int32)
+    vb, vo = W.pack(toks)
+    V = len(toks)
+    h = (T.trie_build_many_device if device_build else T.trie_build_many)(sb, so, si)
+    ov = oracle.Vocab(vb, vo)
+    want = np.concatenate([oracle.mask_all(oracle.Trie(*W.pack(s)), ov) for s in sets])
+    if lists_first:
+        n = T.trie_compile_lists(h, vb, vo, V)
+        assert n == int(np.unpackbits(want.view(np.uint8)).sum())
+    if then == "masks":
+        m = T.alloc_mask(h, V, "cuda")
+        T.trie_compile_masks(h, vb, vo, V, m)
+    else:
+        T.trie_lazy_init(h, vb, vo, V, cache_rows=0, max_batch=h.num_nodes)
+        m = T.trie_lazy_rows(h, torch.arange(h.num_nodes, dtype=torch.int32, device="cuda"), V)
+    assert np.array_equal(m.cpu().numpy().view(np.uint32), want)
+    (h.destroy_async if lists_first else h.destroy)()
