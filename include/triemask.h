@@ -116,15 +116,16 @@ int trie_build_many(const uint8_t *bytes, const int64_t *offsets, const int32_t 
  * of trie_build_many for the same arguments.
  *   Arguments as trie_build_many (all host, read during the call); stream is
  *   the stream the build kernels and the copies run on.
- * The strings are staged on the device and inserted level by level (depth
- * d = 0, 1, ...) for all sets at once; the trie lives on the device only and
+ * The strings are staged on the device and sorted set by set, or, when a set
+ * holds more than 4,096 of them, inserted level by level (depth d = 0, 1, ...)
+ * for all sets at once; the trie lives on the device only and
  * is bound to the current device. Where the device reads pageable host
  * memory coherently through the host's page tables (Grace CPUs over
  * NVLink-C2C), a kernel reads the strings straight from the caller's arrays;
  * elsewhere they are copied first (TRIEMASK_HOST_READ=copy in the
  * environment forces the copies). The offsets are checked on the device.
  * Returns once the node count and the roots are known on the host (read back
- * after the level insertion; the caller's arrays have been read by then):
+ * after the sort or the insertion; the caller's arrays have been read by then):
  * the last kernels (the breadth-first layout and the child links) are still
  * queued on `stream`, so use the handle on `stream` or
  * after synchronising it (calls that copy arrays back synchronise the device
@@ -133,8 +134,9 @@ int trie_build_many(const uint8_t *bytes, const int64_t *offsets, const int32_t 
  * tokens' bytes. Calls that need the host arrays (trie_get_csr,
  * trie_lazy_init) copy them back once. Strings longer than 1024 bytes, more
  * than 2^24 (set, depth) pairs or more than 2^31-3 string bytes plus sets
- * are built by trie_build_many on the host instead. Device scratch (about
- * 20 bytes per string byte plus 90 per string) is taken from the library's
+ * are built by trie_build_many on the host instead. Device scratch
+ * (about 1 byte per string byte plus 20 per string; 20 and 90 when a set holds
+ * more than 4,096 strings) is taken from the library's
  * device memory pool on `stream` and released there. Errors as
  * trie_build_many; TRIE_ENOMEM if a device allocation fails, TRIE_ECUDA if
  * another CUDA call fails. */

@@ -567,7 +567,7 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
     int32_t n = 0, max_len = 0;
     int64_t n_chars = 0;
     cudaError_t e;
-    {
+    try {
         tmk::DeviceBuild db;
         bool ok = true;
         e = db.stage(n_bytes > 0 ? bytes + off[0] : nullptr, off, set_offsets, M, K, n_bytes,
@@ -598,6 +598,8 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
             e = db.emit(const_cast<int32_t *>(h->dev.parent), const_cast<uint8_t *>(h->dev.label),
                         const_cast<uint8_t *>(h->dev.terminal), sms);
         }
+    } catch (const std::bad_alloc &) {
+        e = cudaErrorMemoryAllocation;
     }  // the scratch is freed on the stream after the last kernel
     if (e == cudaSuccess && (rc = finish_device_trie(h, dev, stream)) != TRIE_OK) {
         delete h;

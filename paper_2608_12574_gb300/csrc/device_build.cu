@@ -1,8 +1,9 @@
 // The byte tries of a forest built on the device from the raw strings
 // (Sec. 4.1; App. G.1 Step 1), for per-request sets that change every batch.
 //
-// Level by level over depth d, for all sets at once, without sorting the
-// strings: every string of length > d ORs its byte d into the 256-bit
+// Forests of small sets are sorted set by set (k_b_set_sort, k_b_set_nodes,
+// below). The others: level by level over depth d, for all sets at once,
+// without sorting the strings: every string of length > d ORs its byte d into the 256-bit
 // child-label set of the node it has reached (its parent at depth d); the
 // parents of a level, in order, give their children consecutive ids (first
 // child = the level's end + an exclusive scan of the sets' popcounts), and a
@@ -12,6 +13,7 @@
 // renumbers every node to base(set) + (its rank within the set's own
 // breadth-first order), the layout of the host builder.
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -25,7 +27,12 @@ namespace tmk {
 namespace {
 
 constexpr int kBThreads = 256;
-constexpr int32_t kSetMaxStrings = 4096;  // forests whose sets all hold at most this many strings: one CTA per set
+// Forests whose sets all hold at most this many strings are sorted, one CTA
+// per set (38 B of shared memory a string). 256 sets of 300-2,000 names: 54 us
+// to sort and 30 us to write the nodes, against 178 and 12 us by one CTA per
+// set inserting level by level (seven barriers for each of ~32 levels), and
+// 630 us by the level kernels over all sets.
+constexpr int32_t kSetMaxStrings = 4096;
 constexpr int kScanTile = 1024;  // parents per tile of the level scan
 
 // Staging: copies the strings' offsets, the set offsets and the bytes into
@@ -341,24 +348,16 @@ __global__ void k_b_permute(const int32_t *__restrict__ ls, int32_t D, const int
     }
 }
 
-// ---- Forests of small sets: one CTA per set (kSetThreads threads, each
-// owning up to kSetPer strings), the levels of that set in shared memory. The
-// set's nodes are created in the order of the level path restricted to the
-// set (breadth-first, sorted siblings) at local ids 0, 1, ..., written at
-// ub(s) = (bytes before set s) + s, room for the set's at most 1 + bytes
-// nodes; a scan of the node counts then gives every set its base.
+// ---- Forests of small sets: one CTA per set, without levels. The strings of
+// the set are sorted in shared memory; string i of the sorted order then owns
+// (is the first through) the nodes of depths lcp(i) + 1 .. len(i), lcp(i) the
+// common prefix with string i - 1, so the node count is a sum, and within a
+// depth the nodes in sorted order of their owners are the siblings-sorted
+// breadth-first order: a node's rank is a count of owners before it, found by
+// ballots, with no barrier per level.
 constexpr int kSetThreads = 512;
-constexpr int kSetPer = int(kSetMaxStrings / kSetThreads);
-
-__device__ __forceinline__ int32_t block_reduce_max(int32_t v, int32_t *ws) {
-    v = __reduce_max_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int32_t m = 0;
-    for (int w = 0; w < int(blockDim.x >> 5); w++) m = max(m, ws[w]);
-    __syncthreads();
-    return m;
-}
+constexpr int kSetKeyWords = 4;  // 8-byte words of a string kept in shared memory as its sort key
+constexpr int kSetKeyBytes = 8 * kSetKeyWords;
 
 // Exclusive scan of one int per thread over a block of kSetThreads.
 __device__ __forceinline__ int32_t set_excl_scan(int32_t v, int32_t *ws, int32_t *total) {
@@ -387,121 +386,188 @@ __device__ __forceinline__ int32_t set_excl_scan(int32_t v, int32_t *ws, int32_t
     return before + x - v;
 }
 
-// Dynamic shared memory: the child-label sets of the current level
-// (smax rows of 8 words), for each row the labels counted in its words before
-// each word (8 bytes), the first child of each of its nodes, and a flag per
-// node of the next level that some string ends at.
-__global__ void __launch_bounds__(kSetThreads) k_b_sets(const uint8_t *__restrict__ bytes,
-                                                        const int64_t *__restrict__ off,
-                                                        const int32_t *__restrict__ set_off, int32_t M, int32_t smax,
-                                                        int32_t *__restrict__ parent_ub, uint8_t *__restrict__ label_ub,
-                                                        uint8_t *__restrict__ term_ub, int32_t *__restrict__ count,
-                                                        unsigned long long *__restrict__ chars) {
+// The first min(len, kSetKeyBytes) bytes at p as big-endian words (zeros
+// after them), by the aligned 8-byte words that hold them (all inside the
+// staged image: only words with a byte of the string are read).
+__device__ __forceinline__ void load_key(const uint8_t *p, int32_t len, uint64_t (&w)[kSetKeyWords]) {
+    const int32_t n = len < kSetKeyBytes ? len : kSetKeyBytes;
+    const uint32_t mis = uint32_t(reinterpret_cast<uintptr_t>(p)) & 7u;
+    const uint64_t *q = reinterpret_cast<const uint64_t *>(p - mis);
+    uint64_t raw[kSetKeyWords + 1];
+#pragma unroll
+    for (int k = 0; k <= kSetKeyWords; k++) raw[k] = 8 * k < n + int32_t(mis) && n > 0 ? q[k] : 0ull;
+#pragma unroll
+    for (int k = 0; k < kSetKeyWords; k++) {
+        const uint64_t le = mis ? (raw[k] >> (8 * mis)) | (raw[k + 1] << (64 - 8 * mis)) : raw[k];
+        const uint32_t lo = uint32_t(le), hi = uint32_t(le >> 32);
+        uint64_t be = (uint64_t(__byte_perm(lo, 0, 0x0123)) << 32) | __byte_perm(hi, 0, 0x0123);
+        const int32_t have = n - 8 * k;  // bytes of this word that belong to the string
+        if (have <= 0) be = 0ull;
+        else if (have < 8) be &= ~0ull << (64 - 8 * have);
+        w[k] = be;
+    }
+}
+
+// The strings of one set in shared memory: the key of string j in two halves
+// of 16 bytes (key[j], key[cap + j]: one load compares 16 bytes, and names of
+// one stem agree in their first 8), its length, and its place in the image.
+struct SetStrings {
+    const ulonglong2 *key;
+    int32_t cap;
+    const uint16_t *len;
+    const uint8_t *bytes;
+    const int64_t *off;  // of the set's first string
+    int64_t off0;
+
+    __device__ __forceinline__ uint32_t byte(int32_t j, int32_t k) const { return bytes[off[j] - off0 + k]; }
+
+    // Bytes that strings a and b have in common from their start.
+    __device__ __forceinline__ int32_t common(int32_t a, int32_t b) const {
+        const int32_t n = min(int32_t(len[a]), int32_t(len[b]));
+#pragma unroll
+        for (int h = 0; h < kSetKeyWords / 2; h++) {
+            const ulonglong2 x = key[h * cap + a], y = key[h * cap + b];
+            if (x.x != y.x) return min(n, 16 * h + (__clzll(static_cast<long long>(x.x ^ y.x)) >> 3));
+            if (x.y != y.y) return min(n, 16 * h + 8 + (__clzll(static_cast<long long>(x.y ^ y.y)) >> 3));
+        }
+        int32_t k = min(n, kSetKeyBytes);
+        while (k < n && byte(a, k) == byte(b, k)) k++;
+        return k;
+    }
+
+    // Whether a sorts before b; a0 and b0 are the first halves of their keys.
+    __device__ __forceinline__ bool before(int32_t a, ulonglong2 a0, int32_t b, ulonglong2 b0) const {
+        if (a0.x != b0.x) return a0.x < b0.x;
+        if (a0.y != b0.y) return a0.y < b0.y;
+        const ulonglong2 a1 = key[cap + a], b1 = key[cap + b];
+        if (a1.x != b1.x) return a1.x < b1.x;
+        if (a1.y != b1.y) return a1.y < b1.y;
+        const int32_t la = len[a], lb = len[b], n = min(la, lb);
+        for (int32_t k = kSetKeyBytes; k < n; k++) {
+            const uint32_t x = byte(a, k), y = byte(b, k);
+            if (x != y) return x < y;
+        }
+        return la < lb;  // a prefix, then what it is a prefix of
+    }
+};
+
+// Sorts the strings of every set and gives their order: order[i] (i counted
+// from the set's first string) = {lcp | len << 16, string within the set},
+// the set's node count, and the characters of its distinct strings. Merge sort
+// of 2-byte indices: every thread sorts kSortPer strings, then in each round
+// finds by a search along its output's diagonal where its next kSortPer
+// outputs begin in the two runs, and merges them. Bound by the chain of
+// shared-memory loads of the searches: about 3 us a round at 1,203 strings, 31
+// us in all. (Measured slower: every element searched for by itself in the
+// neighbouring run, four side by side, 68 us for the 256 sets; 8-byte words of
+// the key compared one load after the other, and keys of 32 contiguous bytes,
+// whose first halves share half of the banks, 65 us.) Does nothing when the
+// staging found bad offsets or a string longer than the build takes (flags).
+constexpr int kSortPer = 4;
+
+__global__ void __launch_bounds__(kSetThreads) k_b_set_sort(const uint8_t *__restrict__ bytes,
+                                                            const int64_t *__restrict__ off,
+                                                            const int32_t *__restrict__ set_off, int32_t M,
+                                                            int32_t cap, const int32_t *__restrict__ flags,
+                                                            uint2 *__restrict__ order, int32_t *__restrict__ count,
+                                                            unsigned long long *__restrict__ chars) {
     extern __shared__ uint4 dyn[];
-    uint32_t *bits = reinterpret_cast<uint32_t *>(dyn);
-    uint2 *cum = reinterpret_cast<uint2 *>(bits + int64_t(smax) * 8);
-    int32_t *first = reinterpret_cast<int32_t *>(cum + smax);
-    uint8_t *ends = reinterpret_cast<uint8_t *>(first + smax);
+    ulonglong2 *key = reinterpret_cast<ulonglong2 *>(dyn);
+    uint16_t *len = reinterpret_cast<uint16_t *>(key + 2 * size_t(cap));
+    uint16_t *const ids = len + cap;  // [2 * cap]: the order before and after a round
     __shared__ int32_t ws[kSetThreads / 32];
-    __shared__ int32_t root_term;
     pdl_launch_dependents();
     pdl_wait();
+    if (flags[0] != 0 || flags[1] > kDeviceBuildMaxDepth) return;
     const int tid = threadIdx.x;
-    for (int32_t r = tid; r < smax * 8; r += kSetThreads) bits[r] = 0u;
-    for (int32_t r = tid; r < smax; r += kSetThreads) ends[r] = 0;
+    const int64_t off0 = off[0];
     for (int32_t s = blockIdx.x; s < M; s += gridDim.x) {
-        const int32_t i0 = set_off[s], Ks = set_off[s + 1] - i0;
-        const int64_t ub = off[i0] - off[0] + s;
-        if (tid == 0) root_term = 0;
-        __syncthreads();
-        int32_t st[kSetPer], len[kSetPer], cur[kSetPer], nb[kSetPer];
-        int32_t longest = 0;
-#pragma unroll
-        for (int k = 0; k < kSetPer; k++) {
-            const int32_t j = tid + k * kSetThreads;
-            len[k] = -1;
-            cur[k] = 0;
-            nb[k] = 0;
-            st[k] = 0;
-            if (j < Ks) {
-                const int64_t a = off[i0 + j], e = off[i0 + j + 1];
-                st[k] = int32_t(a - off[0]);
-                len[k] = int32_t(e - a);
-                longest = max(longest, len[k]);
-                if (len[k] == 0) root_term = 1;
-                else nb[k] = bytes[st[k]];
-            }
+        const int32_t i0 = set_off[s], n = set_off[s + 1] - i0;
+        for (int32_t j = tid; j < n; j += kSetThreads) {
+            const int64_t a = off[i0 + j];
+            const int32_t l = int32_t(off[i0 + j + 1] - a);
+            uint64_t w[kSetKeyWords];
+            load_key(bytes + (a - off0), l, w);
+            key[j] = make_ulonglong2(w[0], w[1]);
+            key[cap + j] = make_ulonglong2(w[2], w[3]);
+            len[j] = uint16_t(l);
         }
-        const int32_t dmax = block_reduce_max(longest, ws);  // also orders root_term
+        __syncthreads();
+        const SetStrings str{key, cap, len, bytes, off + i0, off0};
+        uint16_t *src = ids, *dst = ids + cap;
+        for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
+            int32_t x[kSortPer];
+            ulonglong2 x0[kSortPer];
+            const int32_t m = min(kSortPer, n - o);
+#pragma unroll
+            for (int e = 0; e < kSortPer; e++) {
+                x[e] = e < m ? o + e : o;
+                x0[e] = key[x[e]];
+            }
+#pragma unroll
+            for (int r = 1; r < kSortPer; r++)
+#pragma unroll
+                for (int e = r; e > 0; e--)
+                    if (r < m && str.before(x[e], x0[e], x[e - 1], x0[e - 1])) {
+                        const int32_t y = x[e];
+                        const ulonglong2 y0 = x0[e];
+                        x[e] = x[e - 1], x0[e] = x0[e - 1];
+                        x[e - 1] = y, x0[e - 1] = y0;
+                    }
+#pragma unroll
+            for (int e = 0; e < kSortPer; e++)
+                if (e < m) src[o + e] = uint16_t(x[e]);
+        }
+        __syncthreads();
+        for (int32_t w = kSortPer; w < n; w <<= 1) {
+            for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
+                const int32_t first = o & ~(2 * w - 1), diag = o - first;
+                const int32_t na = min(w, n - first), nb = max(0, min(w, n - first - w));
+                const uint16_t *A = src + first, *B = A + w;
+                int32_t lo = max(0, diag - nb), hi = min(diag, na);
+                while (lo < hi) {  // the entries of A among the first diag outputs
+                    const int32_t mid = (lo + hi) >> 1;
+                    const int32_t x = A[mid], y = B[diag - 1 - mid];
+                    if (str.before(y, key[y], x, key[x])) hi = mid;
+                    else lo = mid + 1;
+                }
+                int32_t ia = lo, ib = diag - lo;
+                int32_t x = ia < na ? int32_t(A[ia]) : 0, y = ib < nb ? int32_t(B[ib]) : 0;
+                ulonglong2 x0 = key[x], y0 = key[y];
+#pragma unroll
+                for (int e = 0; e < kSortPer; e++) {
+                    if (o + e >= n) break;
+                    const bool from_b = ib < nb && (ia >= na || str.before(y, y0, x, x0));
+                    dst[o + e] = uint16_t(from_b ? y : x);
+                    if (from_b) {
+                        ib++;
+                        if (ib < nb) y = B[ib], y0 = key[y];
+                    } else {
+                        ia++;
+                        if (ia < na) x = A[ia], x0 = key[x];
+                    }
+                }
+            }
+            __syncthreads();
+            uint16_t *const t = src;
+            src = dst;
+            dst = t;
+        }
+        int32_t nodes = 0, my_chars = 0;
+        for (int32_t i = tid; i < n; i += kSetThreads) {
+            const int32_t b = src[i], l = len[b];
+            const int32_t lcp = i > 0 ? str.common(src[i - 1], b) : 0;
+            order[i0 + i] = make_uint2(uint32_t(lcp) | (uint32_t(l) << 16), uint32_t(b));
+            nodes += l - lcp;
+            if (i == 0 || lcp < l) my_chars += l;  // not a repetition of the string before it
+        }
+        int32_t total, total_chars;
+        set_excl_scan(nodes, ws, &total);
+        set_excl_scan(my_chars, ws, &total_chars);
         if (tid == 0) {
-            parent_ub[ub] = -1;
-            label_ub[ub] = 0;
-            term_ub[ub] = uint8_t(root_term);
+            count[s] = 1 + total;
+            if (total_chars) atomicAdd(chars, static_cast<unsigned long long>(total_chars));
         }
-        int32_t level_start = 0, level_end = 1;
-        unsigned long long my_chars = 0;
-        for (int32_t d = 0; d < dmax; d++) {
-            const int32_t width = level_end - level_start;
-#pragma unroll
-            for (int k = 0; k < kSetPer; k++)
-                if (len[k] > d)
-                    atomicOr(bits + (cur[k] - level_start) * 8 + (nb[k] >> 5), 1u << (nb[k] & 31));
-            __syncthreads();
-            // first child of every node of the level: a contiguous chunk of rows per thread
-            const int32_t per = (width + kSetThreads - 1) / kSetThreads;
-            const int32_t r0 = min(tid * per, width), r1 = min(r0 + per, width);
-            int32_t c = 0;
-            for (int32_t r = r0; r < r1; r++) c += row_popc(bits, r);
-            int32_t total;
-            int32_t at = level_end + set_excl_scan(c, ws, &total);
-            for (int32_t r = r0; r < r1; r++) {
-                const uint4 *rw = reinterpret_cast<const uint4 *>(bits + int64_t(r) * 8);
-                const uint4 lo = rw[0], hi = rw[1];
-                const uint32_t p1 = __popc(lo.x), p2 = p1 + __popc(lo.y), p3 = p2 + __popc(lo.z),
-                               p4 = p3 + __popc(lo.w), p5 = p4 + __popc(hi.x), p6 = p5 + __popc(hi.y),
-                               p7 = p6 + __popc(hi.z);
-                cum[r] = make_uint2((p1 << 8) | (p2 << 16) | (p3 << 24), p4 | (p5 << 8) | (p6 << 16) | (p7 << 24));
-                first[r] = at;
-                at += int32_t(p7 + __popc(hi.w));
-            }
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < kSetPer; k++) {
-                if (len[k] <= d) continue;
-                const uint32_t b = uint32_t(nb[k]);
-                const int32_t row = cur[k] - level_start;
-                const uint32_t wi = b >> 5;
-                const uint2 cm = cum[row];
-                const uint32_t before = ((wi < 4 ? cm.x : cm.y) >> (8 * (wi & 3))) & 0xFFu;
-                const int32_t below = int32_t(before + __popc(bits[row * 8 + wi] & ((1u << (b & 31)) - 1u)));
-                const int32_t ch = first[row] + below;
-                const int64_t g = ub + ch;
-                parent_ub[g] = cur[k];
-                label_ub[g] = uint8_t(b);
-                if (len[k] == d + 1) {
-                    term_ub[g] = 1;
-                    ends[ch - level_end] = 1;
-                } else {
-                    nb[k] = bytes[st[k] + d + 1];
-                }
-                cur[k] = ch;
-            }
-            __syncthreads();
-            for (int32_t r = tid; r < width * 8; r += kSetThreads) bits[r] = 0u;
-            for (int32_t x = tid; x < total; x += kSetThreads)
-                if (ends[x]) {
-                    my_chars += unsigned(d + 1);
-                    ends[x] = 0;
-                }
-            level_start = level_end;
-            level_end += total;
-            __syncthreads();
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) my_chars += __shfl_down_sync(0xffffffffu, my_chars, o);
-        if ((tid & 31) == 0 && my_chars) atomicAdd(chars, my_chars);
-        if (tid == 0) count[s] = level_end;
-        __syncthreads();
     }
 }
 
@@ -527,38 +593,118 @@ __global__ void __launch_bounds__(kBThreads) k_b_set_scan(int32_t M, const int32
     if (threadIdx.x == 0) *total = carry;
 }
 
-// Every set's nodes from ub(s) + i to base(s) + i (kEmitParts CTAs per set,
-// each a share of the set's nodes: one CTA per set left each thread ~70
-// dependent copies at 256 sets of ~19,000 nodes).
-constexpr int32_t kEmitParts = 8;
-__global__ void k_b_set_emit(const int64_t *__restrict__ off, const int32_t *__restrict__ set_off, int32_t M,
-                             const int32_t *__restrict__ count, const int32_t *__restrict__ roots,
-                             const int32_t *__restrict__ parent_ub, const uint8_t *__restrict__ label_ub,
-                             const uint8_t *__restrict__ term_ub, int32_t *__restrict__ parent,
-                             uint8_t *__restrict__ label, uint8_t *__restrict__ terminal) {
+// The nodes of every set from its sorted strings, in their final place: a
+// warp per depth goes through the strings in sorted order, 32 at a time; the
+// owners at that depth take consecutive ids (their stores fall together), and
+// a node's parent is the last owner at the depth above up to its string.
+// kNodesBatch groups of 32 strings at a time, so that their label bytes (from
+// L1 and L2) are waited for once. `parts` CTAs share a set, each taking every
+// parts-th depth.
+constexpr int kNodesBatch = 4;
+
+__global__ void __launch_bounds__(kSetThreads) k_b_set_nodes(const uint8_t *__restrict__ bytes,
+                                                             const int64_t *__restrict__ off,
+                                                             const int32_t *__restrict__ set_off, int32_t M,
+                                                             int32_t cap, int32_t D, int32_t parts,
+                                                             const uint2 *__restrict__ order,
+                                                             const int32_t *__restrict__ roots,
+                                                             int32_t *__restrict__ parent, uint8_t *__restrict__ label,
+                                                             uint8_t *__restrict__ terminal) {
+    extern __shared__ uint4 dyn[];
+    uint2 *str = reinterpret_cast<uint2 *>(dyn);            // sorted: {lcp | len << 16, place in the image}
+    int32_t *start = reinterpret_cast<int32_t *>(str + cap);  // [D + 2] first id of each depth
     pdl_launch_dependents();
     pdl_wait();
-    for (int64_t u = blockIdx.x; u < int64_t(M) * kEmitParts; u += gridDim.x) {
-        const int32_t s = int32_t(u / kEmitParts), part = int32_t(u % kEmitParts);
-        const int64_t ub = off[set_off[s]] - off[0] + s;
-        const int32_t base = roots[s], n = count[s];
-        for (int32_t i = part * int32_t(blockDim.x) + threadIdx.x; i < n; i += kEmitParts * int32_t(blockDim.x)) {
-            const int32_t p = parent_ub[ub + i];
-            parent[base + i] = p < 0 ? -1 : base + p;
-            label[base + i] = label_ub[ub + i];
-            terminal[base + i] = term_ub[ub + i];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t off0 = off[0];
+    for (int64_t u = blockIdx.x; u < int64_t(M) * parts; u += gridDim.x) {
+        const int32_t s = int32_t(u / parts), part = int32_t(u % parts);
+        const int32_t i0 = set_off[s], n = set_off[s + 1] - i0, base = roots[s];
+        __syncthreads();  // the set before this one is done with the shared arrays
+        for (int32_t d = tid; d < D + 2; d += kSetThreads) start[d] = 0;
+        __syncthreads();
+        for (int32_t i = tid; i < n; i += kSetThreads) {
+            const uint2 o = order[i0 + i];
+            const int32_t lcp = int32_t(o.x & 0xFFFFu), l = int32_t(o.x >> 16);
+            str[i] = make_uint2(o.x, uint32_t(off[i0 + int32_t(o.y)] - off0));
+            if (lcp < l) {  // one more owner from depth lcp + 1, one fewer from l + 1
+                atomicAdd(start + lcp + 1, 1);
+                atomicAdd(start + l + 1, -1);
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {  // changes of the owner count -> owners per depth -> first id of each depth
+            int32_t owners = 0, ids = 1;
+            for (int32_t d0 = 1; d0 <= D; d0 += 32) {
+                int32_t x = d0 + lane <= D ? start[d0 + lane] : 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                const int32_t c = owners + x;  // owners at depth d0 + lane
+                int32_t y = d0 + lane <= D ? c : 0;
+                const int32_t mine = y;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t z = __shfl_up_sync(0xffffffffu, y, o);
+                    if (lane >= o) y += z;
+                }
+                if (d0 + lane <= D) start[d0 + lane] = ids + y - mine;
+                owners = __shfl_sync(0xffffffffu, c, 31);
+                ids += __shfl_sync(0xffffffffu, y, 31);
+            }
+        }
+        __syncthreads();
+        if (part == 0 && tid == 0) {
+            parent[base] = -1;
+            label[base] = 0;
+            terminal[base] = n > 0 && (str[0].x >> 16) == 0u;  // the empty string sorts first
+        }
+        for (int32_t d = 1 + warp * parts + part; d <= D; d += (kSetThreads / 32) * parts) {
+            int32_t at = base + start[d];                                // next id at depth d
+            int32_t above = base + (d > 1 ? start[d - 1] - 1 : 0);       // last node seen at depth d - 1
+            for (int32_t c0 = 0; c0 < n; c0 += 32 * kNodesBatch) {
+                int32_t id[kNodesBatch], up[kNodesBatch];
+                uint32_t lab[kNodesBatch];
+                bool ends[kNodesBatch];
+#pragma unroll
+                for (int k = 0; k < kNodesBatch; k++) {
+                    const int32_t i = c0 + 32 * k + lane;
+                    const uint2 sp = i < n ? str[i] : make_uint2(0xFFFFu, 0u);
+                    const int32_t lcp = int32_t(sp.x & 0xFFFFu), l = int32_t(sp.x >> 16);
+                    const bool own = lcp < d && d <= l;
+                    const uint32_t here = __ballot_sync(0xffffffffu, own);
+                    const uint32_t over = __ballot_sync(0xffffffffu, d > 1 && lcp < d - 1 && d - 1 <= l);
+                    id[k] = own ? at + __popc(here & ((1u << lane) - 1u)) : -1;
+                    up[k] = above + __popc(over & (0xFFFFFFFFu >> (31 - lane)));
+                    lab[k] = own ? __ldg(bytes + sp.y + d - 1) : 0u;
+                    ends[k] = d == l;
+                    at += __popc(here);
+                    above += __popc(over);
+                }
+#pragma unroll
+                for (int k = 0; k < kNodesBatch; k++)
+                    if (id[k] >= 0) {
+                        parent[id[k]] = up[k];
+                        label[id[k]] = uint8_t(lab[k]);
+                        terminal[id[k]] = ends[k];
+                    }
+            }
         }
     }
 }
 
 }  // namespace
 
-// Scratch of one device build. Staging part: the strings, level-order node
-// arrays (at most n_bytes + M nodes), two child-label buffers of
-// max(K, M) rows, the level scans, the flags. Level part (once the longest
-// string D is known): the level ends and the (set, depth) tables.
+// Scratch of one device build. Staging part: the strings, the flags and
+// counts read back, and the sorted order of a forest of small sets. Level part
+// (once the longest string D is known): level-order node arrays (at most
+// n_bytes + M nodes), two child-label buffers of max(K, M) rows, the level
+// scans and ends, the (set, depth) tables.
 struct DeviceBuild::Scratch {
     void *base = nullptr, *base2 = nullptr;
+    size_t head_bytes;  // flags, total, characters and roots: one read-back
     uint8_t *bytes;
     uint4 *image;
     int64_t *off;
@@ -566,7 +712,8 @@ struct DeviceBuild::Scratch {
     uint8_t *label_g, *term_g;
     uint32_t *bits[2];
     int32_t *end_sd, *first_sd, *off_sd, *roots, *map;
-    int32_t *count, *total;  // small-set path: nodes per set, all nodes
+    int32_t *count, *total;  // small sets: nodes per set, all nodes
+    uint2 *order;            // small sets: the sorted strings
     unsigned long long *n_chars;
 };
 
@@ -589,6 +736,29 @@ struct Carver {
     }
 };
 
+// What the host reads back in one copy: {bad offsets, longest string, nodes,
+// 0, characters (8 bytes)}, then the roots.
+constexpr size_t kHeadRoots = 24;
+
+size_t sort_smem(int32_t cap) { return size_t(cap) * (kSetKeyBytes + 3 * sizeof(uint16_t)); }
+size_t nodes_smem(int32_t cap, int32_t D) {
+    return size_t(cap) * sizeof(uint2) + sizeof(int32_t) * (size_t(D) + 2);
+}
+
+// Launches a kernel of one CTA per set, at most as many CTAs as are resident
+// at once with `smem` bytes of dynamic shared memory.
+template <typename... Params, typename... Args>
+cudaError_t launch_sets(void (*kernel)(Params...), int64_t sets, size_t smem, int num_sms, cudaStream_t st,
+                        Args... args) {
+    int per_sm = 0;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSetThreads, smem)) != cudaSuccess)
+        return e;
+    const int64_t grid = std::min<int64_t>(sets, int64_t(num_sms) * std::max(per_sm, 1));
+    return launch_pdl_smem(kernel, grid, kSetThreads, smem, st, args...);
+}
+
 }  // namespace
 
 cudaError_t DeviceBuild::stage(const uint8_t *h_bytes, const int64_t *h_off, const int32_t *h_set_off, int32_t M,
@@ -603,45 +773,26 @@ cudaError_t DeviceBuild::stage(const uint8_t *h_bytes, const int64_t *h_off, con
     for (int32_t i = 0; i < M; i++) smax_ = std::max(smax_, h_set_off[i + 1] - h_set_off[i]);
     small_ = smax_ <= kSetMaxStrings;
     s_ = new Scratch();
-    const int64_t U = n_bytes + M;               // nodes at most
-    const int64_t W = std::max<int64_t>(K, M);   // parents of one level at most
-    const int64_t tiles = (W + kScanTile - 1) / kScanTile + 1;
+    s_->head_bytes = kHeadRoots + 4 * size_t(M);
     Carver c;
-    const size_t o_img = c.add(size_t(n_bytes) + 32), o_off = c.add(8 * (size_t(K) + 1)),
-                 o_soff = c.add(4 * (size_t(M) + 1)), o_sset = c.add(4 * size_t(K)), o_cur = c.add(4 * size_t(K)),
-                 o_par = c.add(4 * size_t(U)), o_set = c.add(4 * size_t(U)), o_dep = c.add(4 * size_t(U)),
-                 o_first = c.add(4 * size_t(W)), o_ts = c.add(4 * size_t(tiles)), o_lab = c.add(size_t(U)),
-                 o_term = c.add(size_t(U)), o_b0 = c.add(32 * size_t(W) + 32), o_b1 = c.add(32 * size_t(W) + 32),
-                 o_roots = c.add(4 * size_t(M)), o_map = c.add(4 * size_t(U)), o_nch = c.add(8), o_flags = c.add(8);
+    const size_t o_head = c.add(s_->head_bytes), o_img = c.add(size_t(n_bytes) + 32), o_off = c.add(8 * (size_t(K) + 1)),
+                 o_soff = c.add(4 * (size_t(M) + 1)), o_cnt = c.add(4 * size_t(M)),
+                 o_ord = c.add(small_ ? sizeof(uint2) * size_t(K) : 0);
     cudaError_t e = cudaMallocFromPoolAsync(&s_->base, c.total, pool, st);
     if (e != cudaSuccess) return e;
     char *b = static_cast<char *>(s_->base);
     const size_t mis = reinterpret_cast<uintptr_t>(h_bytes) & 15u;  // the image keeps the source's alignment
+    s_->flags = reinterpret_cast<int32_t *>(b + o_head);
+    s_->total = s_->flags + 2;
+    s_->n_chars = reinterpret_cast<unsigned long long *>(b + o_head + 16);
+    s_->roots = reinterpret_cast<int32_t *>(b + o_head + kHeadRoots);
     s_->image = reinterpret_cast<uint4 *>(b + o_img);
     s_->bytes = reinterpret_cast<uint8_t *>(b + o_img) + mis;
     s_->off = reinterpret_cast<int64_t *>(b + o_off);
     s_->set_off = reinterpret_cast<int32_t *>(b + o_soff);
-    s_->str_set = reinterpret_cast<int32_t *>(b + o_sset);
-    s_->cur = reinterpret_cast<int32_t *>(b + o_cur);
-    s_->parent_g = reinterpret_cast<int32_t *>(b + o_par);
-    s_->set_g = reinterpret_cast<int32_t *>(b + o_set);
-    s_->depth_g = reinterpret_cast<int32_t *>(b + o_dep);
-    s_->first = reinterpret_cast<int32_t *>(b + o_first);
-    s_->tile_sum = reinterpret_cast<int32_t *>(b + o_ts);
-    s_->label_g = reinterpret_cast<uint8_t *>(b + o_lab);
-    s_->term_g = reinterpret_cast<uint8_t *>(b + o_term);
-    s_->bits[0] = reinterpret_cast<uint32_t *>(b + o_b0);
-    s_->bits[1] = reinterpret_cast<uint32_t *>(b + o_b1);
-    s_->roots = reinterpret_cast<int32_t *>(b + o_roots);
-    s_->map = reinterpret_cast<int32_t *>(b + o_map);
-    s_->n_chars = reinterpret_cast<unsigned long long *>(b + o_nch);
-    s_->flags = reinterpret_cast<int32_t *>(b + o_flags);
-    if ((e = cudaMemsetAsync(s_->term_g, 0, size_t(U), st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s_->bits[0], 0, 32 * size_t(W) + 32, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s_->bits[1], 0, 32 * size_t(W) + 32, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s_->n_chars, 0, 8, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(s_->flags, 0, 8, st)) != cudaSuccess)
-        return e;
+    s_->count = reinterpret_cast<int32_t *>(b + o_cnt);
+    s_->order = reinterpret_cast<uint2 *>(b + o_ord);
+    if ((e = cudaMemsetAsync(s_->flags, 0, kHeadRoots, st)) != cudaSuccess) return e;
     const int64_t n_vec = n_bytes > 0 ? (int64_t(mis) + n_bytes + 15) / 16 : 0;
     const int64_t items = std::max<int64_t>(std::max<int64_t>(K, M) + 1, n_vec);
     const int64_t grid = std::min<int64_t>((items + kBThreads - 1) / kBThreads, int64_t(num_sms) * 16);
@@ -660,13 +811,32 @@ cudaError_t DeviceBuild::stage(const uint8_t *h_bytes, const int64_t *h_off, con
                    s_->off, s_->set_off, s_->image, s_->flags);
     }
     if (e != cudaSuccess) return e;
-    int32_t flags[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(flags, s_->flags, sizeof(flags), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    if (small_ &&
+        ((e = launch_sets(k_b_set_sort, M, sort_smem(smax_), num_sms, st, static_cast<const uint8_t *>(s_->bytes),
+                          static_cast<const int64_t *>(s_->off), static_cast<const int32_t *>(s_->set_off), M, smax_,
+                          static_cast<const int32_t *>(s_->flags), s_->order, s_->count, s_->n_chars)) !=
+             cudaSuccess ||
+         (e = launch_pdl(k_b_set_scan, 1, kBThreads, st, M, static_cast<const int32_t *>(s_->count), s_->roots,
+                         s_->total)) != cudaSuccess))
         return e;
-    *offsets_ok = flags[0] == 0;
-    *max_len = flags[1];
+    if ((e = read_head()) != cudaSuccess) return e;
+    *offsets_ok = head_[0] == 0;
+    *max_len = head_[1];
     return cudaSuccess;
+}
+
+// The flags, counts and roots, in one copy (host-synchronous).
+cudaError_t DeviceBuild::read_head() {
+    head_.resize(s_->head_bytes / 4);
+    const cudaError_t e = cudaMemcpyAsync(head_.data(), s_->flags, s_->head_bytes, cudaMemcpyDeviceToHost, stream_);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(stream_);
+}
+
+void DeviceBuild::take_head(int32_t *n_nodes, std::vector<int32_t> *roots, int64_t *n_chars) {
+    n_ = head_[2];
+    *n_nodes = n_;
+    memcpy(n_chars, head_.data() + 4, sizeof(int64_t));
+    roots->assign(head_.begin() + kHeadRoots / 4, head_.end());
 }
 
 cudaError_t DeviceBuild::levels(int32_t D, int num_sms, int32_t *n_nodes, std::vector<int32_t> *roots,
@@ -674,21 +844,41 @@ cudaError_t DeviceBuild::levels(int32_t D, int num_sms, int32_t *n_nodes, std::v
     const cudaStream_t st = stream_;
     const int32_t M = M_, K = K_;
     D_ = D;
-    if (small_) return sets(num_sms, n_nodes, roots, n_chars);
-    const int64_t U = n_bytes_ + M;
-    const int64_t W = std::max<int64_t>(K, M);
+    if (small_) {  // sorted and counted behind the staging
+        take_head(n_nodes, roots, n_chars);
+        return cudaSuccess;
+    }
+    const int64_t U = n_bytes_ + M;             // nodes at most
+    const int64_t W = std::max<int64_t>(K, M);  // parents of one level at most
+    const int64_t tiles = (W + kScanTile - 1) / kScanTile + 1;
     const int64_t sd = int64_t(M) * (D + 1);
     Carver c;
-    const size_t o_ls = c.add(4 * (size_t(D) + 2)), o_end = c.add(4 * size_t(sd)), o_fsd = c.add(4 * size_t(sd)),
-                 o_osd = c.add(4 * size_t(sd));
+    const size_t o_term = c.add(size_t(U)), o_b0 = c.add(32 * size_t(W) + 32), o_b1 = c.add(32 * size_t(W) + 32),
+                 o_end = c.add(4 * size_t(sd)), zeroed = c.total, o_sset = c.add(4 * size_t(K)),
+                 o_cur = c.add(4 * size_t(K)), o_par = c.add(4 * size_t(U)), o_set = c.add(4 * size_t(U)),
+                 o_dep = c.add(4 * size_t(U)), o_first = c.add(4 * size_t(W)), o_ts = c.add(4 * size_t(tiles)),
+                 o_lab = c.add(size_t(U)), o_map = c.add(4 * size_t(U)), o_ls = c.add(4 * (size_t(D) + 2)),
+                 o_fsd = c.add(4 * size_t(sd)), o_osd = c.add(4 * size_t(sd));
     cudaError_t e = cudaMallocFromPoolAsync(&s_->base2, c.total, pool_, st);
     if (e != cudaSuccess) return e;
     char *b = static_cast<char *>(s_->base2);
-    s_->ls = reinterpret_cast<int32_t *>(b + o_ls);
+    s_->term_g = reinterpret_cast<uint8_t *>(b + o_term);
+    s_->bits[0] = reinterpret_cast<uint32_t *>(b + o_b0);
+    s_->bits[1] = reinterpret_cast<uint32_t *>(b + o_b1);
     s_->end_sd = reinterpret_cast<int32_t *>(b + o_end);
+    s_->str_set = reinterpret_cast<int32_t *>(b + o_sset);
+    s_->cur = reinterpret_cast<int32_t *>(b + o_cur);
+    s_->parent_g = reinterpret_cast<int32_t *>(b + o_par);
+    s_->set_g = reinterpret_cast<int32_t *>(b + o_set);
+    s_->depth_g = reinterpret_cast<int32_t *>(b + o_dep);
+    s_->first = reinterpret_cast<int32_t *>(b + o_first);
+    s_->tile_sum = reinterpret_cast<int32_t *>(b + o_ts);
+    s_->label_g = reinterpret_cast<uint8_t *>(b + o_lab);
+    s_->map = reinterpret_cast<int32_t *>(b + o_map);
+    s_->ls = reinterpret_cast<int32_t *>(b + o_ls);
     s_->first_sd = reinterpret_cast<int32_t *>(b + o_fsd);
     s_->off_sd = reinterpret_cast<int32_t *>(b + o_osd);
-    if ((e = cudaMemsetAsync(s_->end_sd, 0, 4 * size_t(sd), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(b, 0, zeroed, st)) != cudaSuccess) return e;
     const int64_t sgrid = (W + kBThreads - 1) / kBThreads;
     if ((e = launch_pdl(k_b_init, sgrid, kBThreads, st, static_cast<const uint8_t *>(s_->bytes),
                     static_cast<const int64_t *>(s_->off), static_cast<const int32_t *>(s_->set_off), M, K,
@@ -721,77 +911,24 @@ cudaError_t DeviceBuild::levels(int32_t D, int num_sms, int32_t *n_nodes, std::v
                     static_cast<const int32_t *>(s_->first_sd), static_cast<const int32_t *>(s_->off_sd), s_->map)) !=
             cudaSuccess)
         return e;
-    // the node count, the roots and the characters (host-synchronous)
-    int32_t n = 0;
-    unsigned long long nc = 0;
-    roots->resize(size_t(M));
-    if ((e = cudaMemcpyAsync(&n, s_->ls + D + 1, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(roots->data(), s_->roots, 4 * size_t(M), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&nc, s_->n_chars, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    // the node count beside the roots and the characters
+    if ((e = cudaMemcpyAsync(s_->total, s_->ls + D + 1, 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
+        (e = read_head()) != cudaSuccess)
         return e;
-    *n_nodes = n;
-    *n_chars = int64_t(nc);
-    n_ = n;
-    return cudaSuccess;
-}
-
-cudaError_t DeviceBuild::sets(int num_sms, int32_t *n_nodes, std::vector<int32_t> *roots, int64_t *n_chars) {
-    const cudaStream_t st = stream_;
-    const int32_t M = M_;
-    Carver c;
-    const size_t o_cnt = c.add(4 * size_t(M)), o_tot = c.add(4);
-    cudaError_t e = cudaMallocFromPoolAsync(&s_->base2, c.total, pool_, st);
-    if (e != cudaSuccess) return e;
-    char *b = static_cast<char *>(s_->base2);
-    s_->count = reinterpret_cast<int32_t *>(b + o_cnt);
-    s_->total = reinterpret_cast<int32_t *>(b + o_tot);
-    const size_t smem = size_t(smax_) * (8 * sizeof(uint32_t) + sizeof(uint2) + sizeof(int32_t) + 1);
-    int per_sm = 0;
-    if ((e = cudaFuncSetAttribute(k_b_sets, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) !=
-            cudaSuccess ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_b_sets, kSetThreads, smem)) != cudaSuccess)
-        return e;
-    const int64_t grid = std::min<int64_t>(M, int64_t(num_sms) * std::max(per_sm, 1));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(unsigned(kSetThreads));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if ((e = cudaLaunchKernelEx(&cfg, k_b_sets, static_cast<const uint8_t *>(s_->bytes),
-                                static_cast<const int64_t *>(s_->off), static_cast<const int32_t *>(s_->set_off), M,
-                                smax_, s_->parent_g, s_->label_g, s_->term_g, s_->count, s_->n_chars)) !=
-            cudaSuccess ||
-        (e = launch_pdl(k_b_set_scan, 1, kBThreads, st, M, static_cast<const int32_t *>(s_->count), s_->roots,
-                    s_->total)) != cudaSuccess)
-        return e;
-    int32_t n = 0;
-    unsigned long long nc = 0;
-    roots->resize(size_t(M));
-    if ((e = cudaMemcpyAsync(&n, s_->total, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(roots->data(), s_->roots, 4 * size_t(M), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&nc, s_->n_chars, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-        return e;
-    *n_nodes = n;
-    *n_chars = int64_t(nc);
-    n_ = n;
+    take_head(n_nodes, roots, n_chars);
     return cudaSuccess;
 }
 
 cudaError_t DeviceBuild::emit(int32_t *parent, uint8_t *label, uint8_t *terminal, int num_sms) {
-    if (small_)
-        return launch_pdl(k_b_set_emit, std::min<int64_t>(int64_t(M_) * kEmitParts, int64_t(num_sms) * 16), kBThreads,
-                          stream_,
-                      static_cast<const int64_t *>(s_->off), static_cast<const int32_t *>(s_->set_off), M_,
-                      static_cast<const int32_t *>(s_->count), static_cast<const int32_t *>(s_->roots),
-                      static_cast<const int32_t *>(s_->parent_g), static_cast<const uint8_t *>(s_->label_g),
-                      static_cast<const uint8_t *>(s_->term_g), parent, label, terminal);
+    if (small_) {
+        // a few sets: their depths over several CTAs each, up to four CTAs an SM
+        const int32_t parts = int32_t(std::min<int64_t>(8, std::max<int64_t>(1, 4 * int64_t(num_sms) / M_)));
+        return launch_sets(k_b_set_nodes, int64_t(M_) * parts, nodes_smem(smax_, D_), num_sms, stream_,
+                           static_cast<const uint8_t *>(s_->bytes), static_cast<const int64_t *>(s_->off),
+                           static_cast<const int32_t *>(s_->set_off), M_, smax_, D_, parts,
+                           static_cast<const uint2 *>(s_->order), static_cast<const int32_t *>(s_->roots), parent,
+                           label, terminal);
+    }
     const int64_t ngrid = std::min<int64_t>((int64_t(n_) + kBThreads - 1) / kBThreads, int64_t(num_sms) * 16);
     return launch_pdl(k_b_permute, ngrid, kBThreads, stream_, static_cast<const int32_t *>(s_->ls), D_,
                   static_cast<const int32_t *>(s_->map), static_cast<const int32_t *>(s_->parent_g),

@@ -347,9 +347,10 @@ struct DevLazy {
 
 // A forest built on the device (device_build.cu): stage() copies the strings
 // into its own scratch (reading the caller's host memory directly when
-// `direct`), checks their offsets and returns the longest string's length
-// (host-synchronous); levels() runs the level loop and the renumbering and
-// returns the node count, the roots and the characters (host-synchronous);
+// `direct`), checks their offsets, sorts small sets, and returns the longest
+// string's length (host-synchronous); levels() returns the node count, the
+// roots and the characters, after the level loop and the renumbering when a
+// set is not small (then host-synchronous);
 // emit() writes parent, label and terminal of the final layout into the
 // caller's device arrays (asynchronous); the destructor frees the scratch on
 // the stream after them.
@@ -368,15 +369,16 @@ public:
     cudaError_t emit(int32_t *parent, uint8_t *label, uint8_t *terminal, int num_sms);
 
 private:
-    // forests of small sets: one CTA per set (called by levels())
-    cudaError_t sets(int num_sms, int32_t *n_nodes, std::vector<int32_t> *roots, int64_t *n_chars);
+    cudaError_t read_head();
+    void take_head(int32_t *n_nodes, std::vector<int32_t> *roots, int64_t *n_chars);
     struct Scratch;
     Scratch *s_ = nullptr;
     cudaStream_t stream_ = nullptr;
     cudaMemPool_t pool_ = nullptr;
     int32_t M_ = 0, K_ = 0, D_ = 0, n_ = 0;
     int32_t smax_ = 1;    // strings of the largest set
-    bool small_ = false;  // one CTA per set
+    bool small_ = false;  // every set sorted by one CTA
+    std::vector<int32_t> head_;  // the flags, counts and roots read back
     int64_t n_bytes_ = 0;
 };
 

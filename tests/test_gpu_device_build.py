@@ -374,3 +374,26 @@ def test_child_links_walk_every_byte(cuda, builder):
     assert np.array_equal(got, child)
     assert int(err.item()) == int((child == T.TRIE_STATE_DEAD).sum())
     h.destroy()
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 511, 513, 2048, 2049, 4096])
+def test_device_forest_sorted_sets(cuda, n):
+    """Sets that one CTA sorts, at the edges of its merge rounds and of its
+    threads' shares: strings that agree in their first 8, 16, 32 and more
+    bytes (the words of the sort key, and past them), trailing zero bytes
+    against shorter strings, prefixes, repetitions and the empty string."""
+    r = random.Random(n)
+    stem = bytes(r.randrange(97, 100) for _ in range(60))
+    pick = [lambda: stem[:r.choice([7, 8, 9, 15, 16, 24, 31, 32, 33, 40, 60])],
+            lambda: bytes(r.choice([0, 1, 255]) for _ in range(r.randrange(0, 3))),
+            lambda: stem[:r.choice([8, 32, 33])] + b"\0" * r.randrange(0, 3),
+            lambda: bytes(r.randrange(256) for _ in range(r.randrange(1, 12)))]
+    big = [r.choice(pick)() + r.choice(pick)() for _ in range(n)]
+    sets = [[], big, [b""], big[: n // 2] + big[: n // 3], [stem + stem]]
+    sb, so, index = _forest(sets)
+    h = T.trie_build_many_device(sb, so, index)
+    _check_against_oracle(h, sets)
+    host = T.trie_build_many(sb, so, index)
+    for k, v in host.csr().items():
+        assert np.array_equal(h.csr()[k], v), k
+    assert h.num_chars == host.num_chars and h.max_depth == host.max_depth
