@@ -1310,13 +1310,15 @@ __global__ void k_rt_insert(const int32_t *__restrict__ parent, const uint8_t *_
 // nodes' ancestors are neighbours, so these loads fall together and come from
 // L1 and L2, where reading each entry's row from the 64-byte ancestor rows of
 // the dense compile's tables was 305 MB of DRAM reads a walk on the 4.77 M-node
-// forest (count walk 132 us, 104 us so; write walk 177 and 143 us; and the
-// forest needs no such tables). Called by whole warps, whose lanes stay
+// forest (count walk 132 us, 98 us so; write walk 177 and 139 us; and the
+// forest needs no such tables). Bound by the L1's look-ups of the random edge
+// slots (two, three or four nodes a lane, their loads side by side: 272, 381
+// and 376 us for both walks and the scan, 264 us with one). Called by whole warps, whose lanes stay
 // together until the longest walk ends: with a return at each lane's own end
 // the lanes ran on one by one (326 and 520 us).
 template <typename Tok>
 __device__ __forceinline__ void walk_node(const WalkArgs &a, const int2 *root, int32_t m, Tok tok) {
-    int32_t p = -1, x = -1, t = -1;
+    int32_t p = -1, x = -1, t = -1;  // (x, t): the edge taken by the label below p
     uint32_t c = 0u;
     if (m < a.n_nodes) {
         p = __ldg(a.parent + m);
@@ -1326,17 +1328,28 @@ __device__ __forceinline__ void walk_node(const WalkArgs &a, const int2 *root, i
         t = root[c].y;
     }
     bool on = p >= 0 && x >= 0;
-    while (__any_sync(0xffffffffu, on)) {  // (x, t): the edge taken by the label below p
+    while (__any_sync(0xffffffffu, on)) {
         const int32_t row = p;
+        uint32_t key = 0u, slot = 0u;
+        uint4 e = make_uint4(0u, 0u, 0u, 0u);
+        bool up = false;
         if (on) {
             p = __ldg(a.parent + row);
             c = __ldg(a.label + row);
+            key = ((uint32_t(x) << 8) | c) + 1u;
+            slot = edge_slot(key, a.edge_shift);
+            up = p >= 0;
+            if (up) e = __ldg(a.edge + slot);  // in flight while the entry is emitted
             if (t >= 0) tok(row, t, m);
-            uint4 e;
-            on = p >= 0 && rt_step(a.edge, a.edge_mask, a.edge_shift, x, c, &e);
-            x = int32_t(e.y);
-            t = int32_t(e.z);
         }
+        // the table is at most half full, so an empty slot ends every probe sequence
+        for (uint32_t i = 0; e.x != key && e.x != 0u && i < a.edge_mask; i++) {
+            slot = (slot + 1u) & a.edge_mask;
+            e = __ldg(a.edge + slot);
+        }
+        on = up && e.x == key;
+        x = int32_t(e.y);
+        t = int32_t(e.z);
     }
 }
 
