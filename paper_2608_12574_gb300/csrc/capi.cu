@@ -1265,14 +1265,11 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     const size_t o_stamp = lay.add(sizeof(uint32_t) * size_t(C));
     const size_t o_ctrl = lay.add(sizeof(tmk::LazyCtrl));
     const size_t o_slot = lay.add(sizeof(int32_t) * mb);
-    const size_t o_mnode = lay.add(sizeof(int32_t) * mb);
-    const size_t o_mslot = lay.add(sizeof(int32_t) * mb);
-    const size_t o_rowu = lay.add(sizeof(int32_t) * mb);
-    const size_t o_task = lay.add(sizeof(int4) * (mb + size_t(tmk::kLazySplitRows) * tmk::kLazyMaxParts));
+    const size_t o_task = lay.add(sizeof(tmk::LazyTask) * (mb + size_t(tmk::kLazySplitRows) * tmk::kLazyMaxParts));
     const size_t o_pnode = lay.add(sizeof(int32_t) * n);
     const size_t o_pdep = lay.add(sizeof(int32_t) * n);
     const size_t o_psize = lay.add(sizeof(int32_t) * n);
-    const size_t o_pos = lay.add(sizeof(int32_t) * n);
+    const size_t o_place = lay.add(sizeof(int2) * n);
     const size_t o_pre = lay.add(sizeof(tmk::LazyNode) * n);
     void *base = nullptr;
     if ((rc = pool_alloc(dev, lay.total, 0, &base, "the lazy rows")) != TRIE_OK) return rc;
@@ -1288,14 +1285,11 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     L.stamp = reinterpret_cast<uint32_t *>(b + o_stamp);
     L.ctrl = reinterpret_cast<tmk::LazyCtrl *>(b + o_ctrl);
     L.slot_of = reinterpret_cast<int32_t *>(b + o_slot);
-    L.miss_node = reinterpret_cast<int32_t *>(b + o_mnode);
-    L.miss_slot = reinterpret_cast<int32_t *>(b + o_mslot);
-    L.row_u = reinterpret_cast<int32_t *>(b + o_rowu);
-    L.task = reinterpret_cast<int4 *>(b + o_task);
+    L.task = reinterpret_cast<tmk::LazyTask *>(b + o_task);
     L.pre_node = reinterpret_cast<int32_t *>(b + o_pnode);
     L.pre_depth = reinterpret_cast<int32_t *>(b + o_pdep);
     L.pre_size = reinterpret_cast<int32_t *>(b + o_psize);
-    L.pos_of = reinterpret_cast<int32_t *>(b + o_pos);
+    L.place = reinterpret_cast<int2 *>(b + o_place);
     L.pre = reinterpret_cast<tmk::LazyNode *>(b + o_pre);
     const tmk::LazyCtrl ctrl0 = {1u, 0, 0, 0, 0ull, 0ull};
     const tmk::HostTrie &t = h->host;

@@ -217,6 +217,27 @@ __device__ __forceinline__ uint32_t byte_at(const uint32_t (&w)[4], int32_t i) {
     return (v >> ((i & 3) * 8)) & 0xFFu;
 }
 
+// Whether the token bytes t (zero-padded to 16), k <= 16 of them, are the last
+// k labels of a window (byte i = the label i levels up): token byte j must
+// equal label k - 1 - j, so the token's 16 bytes are reversed and shifted down
+// by 16 - k, which brings byte k - 1 down to byte 0. (Byte by byte, each a
+// select from four registers on either side, the comparison was a good part of
+// the searches' instructions: 8 lazy steps at K = 10,000, B = 256, 217.0 us,
+// 207.6 us so; the compile kernels, whose search runs beside the fill,
+// 505.1 us to 501.3 us at K = 74,719.)
+__device__ __forceinline__ bool spells_window(const uint32_t (&lab)[4], const uint4 t, int32_t k) {
+    const uint64_t win_lo = lab[0] | (uint64_t(lab[1]) << 32), win_hi = lab[2] | (uint64_t(lab[3]) << 32);
+    const uint64_t r_lo = __byte_perm(t.w, 0, 0x0123) | (uint64_t(__byte_perm(t.z, 0, 0x0123)) << 32);
+    const uint64_t r_hi = __byte_perm(t.y, 0, 0x0123) | (uint64_t(__byte_perm(t.x, 0, 0x0123)) << 32);
+    if (k <= 8) {  // label bytes 0..k-1, all from the first half of the token
+        const int s = 8 * (8 - k);
+        return ((r_hi >> s) ^ (win_lo << s >> s)) == 0ull;
+    }
+    const int s = 8 * (16 - k);  // 0..56
+    const uint64_t x_lo = s ? (r_lo >> s) | (r_hi << (64 - s)) : r_lo;
+    return x_lo == win_lo && (r_hi >> s) == (win_hi << s >> s);
+}
+
 // Calls hit(t) for every token id t stored under `key` whose bytes equal the
 // k-edge path ending at node m. lab (if not null) holds the path's labels,
 // byte i = label of the edge i levels above m; otherwise the path is walked
@@ -480,13 +501,7 @@ __device__ __forceinline__ void wavefront(const PatchArgs &a, int32_t m, int k0,
         if (slow & (1u << i)) {
             probe(a, key[i], k, &lab, m, [&](int32_t t) { hit(i, anc_at(an, k - 1), t); });
         } else if (tlen[i] == k) {
-            // token byte j must equal the label k-1-j levels above m
-            const uint32_t tw[4] = {tb[i].x, tb[i].y, tb[i].z, tb[i].w};
-            bool eq = true;
-#pragma unroll
-            for (int j = 0; j < kMaxClimb; j++)
-                if (j < k) eq = eq && byte_at(tw, j) == byte_at(lab, k - 1 - j);
-            if (eq) hit(i, anc_at(an, k - 1), tid[i]);
+            if (spells_window(lab, tb[i], k)) hit(i, anc_at(an, k - 1), tid[i]);
         }
     }
 }
@@ -1485,14 +1500,8 @@ struct LazyArgs {
     uint32_t *stamp;
     LazyCtrl *ctrl;
     int32_t *slot_of;
-    int32_t *miss_node;
-    int32_t *miss_slot;
-    int32_t *row_u;
-    int4 *task;
-    const int32_t *pre_node;
-    const int32_t *pre_depth;
-    const int32_t *pre_size;
-    const int32_t *pos_of;
+    LazyTask *task;
+    const int2 *place;
     const LazyNode *pre;
     int32_t C;        // cache rows
     int32_t n_sets;   // C / kLazyWays
@@ -1503,7 +1512,6 @@ struct LazyArgs {
 
 constexpr int kResolveThreads = 1024;
 constexpr int kLazyRowThreads = 256;
-constexpr int32_t kPending = -3;
 
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     x ^= x >> 16;
@@ -1519,26 +1527,33 @@ __device__ __forceinline__ int32_t lazy_set(int32_t s, int32_t n_sets) {
 }
 
 // Cache tags and stamps are read through L2 (ld.global.cg): other threads of
-// the CTA change them with atomics during the kernel.
+// the CTA change them with atomics during the kernel. Bound by its chain of
+// dependent loads, one after the other: state and token, the move, the tags,
+// and for a missing node its place and stamps (both at once) and the claim; a
+// thread keeps its batch rows' results in registers and the missing nodes stay
+// in shared memory, so nothing is passed on through L2 between the phases
+// (K = 10,000, B = 256, no cache: 6.7-7.1 us of a step from the apply before
+// to its end, 4.6-6.4 us so).
+constexpr int kResolvePer = kLazyMaxBatch / kResolveThreads;  // batch rows per thread
+
 template <bool kAdvance>
 __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, AdvanceArgs aa,
                                                                   const int32_t *states_in,
                                                                   const int32_t *__restrict__ tokens,
                                                                   int32_t *states_out, int32_t *__restrict__ err,
                                                                   int32_t B) {
-    extern __shared__ int32_t sh[];  // [uniq] node keys, [uniq] their miss index
+    extern __shared__ int32_t sh[];  // [uniq] node keys, [uniq] their cache rows
     int32_t *keys = sh;
     int32_t *vals = sh + L.uniq;
-    __shared__ int32_t n_u, n_tasks, n_split;
+    __shared__ int32_t n_u, n_tasks, n_split, n_hit, n_miss_rows;
     __shared__ int32_t split_slot[kLazySplitRows];
-    __shared__ unsigned long long n_hit, n_miss_rows;
     for (int32_t i = threadIdx.x; i < L.uniq; i += blockDim.x) keys[i] = -1;
     if (threadIdx.x == 0) {
         n_u = 0;
         n_tasks = 0;
         n_split = 0;
-        n_hit = 0ull;
-        n_miss_rows = 0ull;
+        n_hit = 0;
+        n_miss_rows = 0;
     }
     __syncthreads();
     pdl_launch_dependents();
@@ -1546,7 +1561,13 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
     const uint32_t now = __ldcg(&L.ctrl->now);
     const uint32_t umask = uint32_t(L.uniq - 1);
     // 1. states; cache lookups; distinct missing nodes into the table
-    for (int32_t b = threadIdx.x; b < B; b += blockDim.x) {
+    int32_t slot[kResolvePer], at[kResolvePer];  // the batch row's cache row; its node's place in the table
+#pragma unroll
+    for (int q = 0; q < kResolvePer; q++) {
+        const int32_t b = threadIdx.x + q * kResolveThreads;
+        slot[q] = -1;  // the {EOS} row
+        at[q] = -1;
+        if (b >= B) continue;
         int32_t s;
         if (kAdvance) {
             const int32_t s0 = states_in[b];
@@ -1556,49 +1577,42 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
         } else {
             s = states_in[b];
         }
-        int32_t slot = -1;  // the {EOS} row
-        if (s >= 0 && s < L.n_nodes) {
-            const int32_t base = (L.n_sets > 0 ? lazy_set(s, L.n_sets) : 0) * kLazyWays;
-            int32_t hit = -1;
-            if (L.n_sets > 0) {
+        if (s < 0 || s >= L.n_nodes) continue;
+        int32_t hit = -1;
+        if (L.n_sets > 0) {
+            const int32_t base = lazy_set(s, L.n_sets) * kLazyWays;
+            const int4 *tags = reinterpret_cast<const int4 *>(L.tag + base);
+            const int4 lo = __ldcg(tags), hi = __ldcg(tags + 1);
+            const int32_t tag[kLazyWays] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
-                for (int w = 0; w < kLazyWays; w++)
-                    if (__ldcg(L.tag + base + w) == s) hit = base + w;
-            }
-            if (hit >= 0) {
-                L.stamp[hit] = now;
-                slot = hit;
-                atomicAdd(&n_hit, 1ull);
-            } else {
-                uint32_t h = mix32(uint32_t(s)) & umask;
-                for (uint32_t it = 0; it <= umask; it++) {  // the table holds >= 2 B slots
-                    const int32_t k = atomicCAS(keys + h, -1, s);
-                    if (k == -1 || k == s) break;
-                    h = (h + 1u) & umask;
-                }
-                L.row_u[b] = int32_t(h);
-                slot = kPending;
-                atomicAdd(&n_miss_rows, 1ull);
-            }
+            for (int w = 0; w < kLazyWays; w++)
+                if (tag[w] == s) hit = base + w;
         }
-        L.slot_of[b] = slot;
+        if (hit >= 0) {
+            L.stamp[hit] = now;
+            slot[q] = hit;
+            atomicAdd(&n_hit, 1);
+        } else {
+            uint32_t h = mix32(uint32_t(s)) & umask;
+            for (uint32_t it = 0; it <= umask; it++) {  // the table holds >= 2 B slots
+                const int32_t k = atomicCAS(keys + h, -1, s);
+                if (k == -1 || k == s) break;
+                h = (h + 1u) & umask;
+            }
+            at[q] = int32_t(h);
+            atomicAdd(&n_miss_rows, 1);
+        }
     }
     __syncthreads();
-    // 2. number the distinct missing nodes
+    // 2. a row for each distinct missing node: the least recently used row of
+    // its set that this call does not use, claimed by a compare-and-swap of its
+    // stamp, else a per-call row; and its tasks
     for (int32_t i = threadIdx.x; i < L.uniq; i += blockDim.x) {
-        const int32_t k = keys[i];
-        if (k >= 0) {
-            const int32_t u = atomicAdd(&n_u, 1);
-            vals[i] = u;
-            L.miss_node[u] = k;
-        }
-    }
-    __syncthreads();
-    // 3. a row for each: the least recently used row of its set that this call
-    // does not use, claimed by a compare-and-swap of its stamp
-    for (int32_t u = threadIdx.x; u < n_u; u += blockDim.x) {
-        const int32_t s = L.miss_node[u];
-        int32_t slot = L.C + u;  // per-call row
+        const int32_t s = keys[i];
+        if (s < 0) continue;
+        const int2 place = __ldg(L.place + s);
+        const int32_t u = atomicAdd(&n_u, 1);
+        int32_t row = L.C + u;  // per-call row
         if (L.n_sets > 0) {
             const int32_t base = lazy_set(s, L.n_sets) * kLazyWays;
             for (int att = 0; att < 4 * kLazyWays; att++) {
@@ -1614,27 +1628,39 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
                 }
                 if (best < 0) break;
                 if (atomicCAS(L.stamp + base + best, best_st, now) == best_st) {
-                    slot = base + best;
-                    L.tag[slot] = s;
+                    row = base + best;
+                    L.tag[row] = s;
                     break;
                 }
             }
         }
-        L.miss_slot[u] = slot;
+        vals[i] = row;
         // CTA tasks: one, or up to kLazyMaxParts for a large subtree (for the
         // first kLazySplitRows such rows of the call)
-        const int32_t desc = __ldg(L.pre_size + __ldg(L.pos_of + s)) - 1;
+        const int32_t desc = place.y - 1;
         int32_t parts = 1;
         if (desc > kLazyPartNodes) {
-            const int32_t i = atomicAdd(&n_split, 1);
-            if (i < kLazySplitRows) {
+            const int32_t j = atomicAdd(&n_split, 1);
+            if (j < kLazySplitRows) {
                 parts = (desc + kLazyPartNodes - 1) / kLazyPartNodes;
                 parts = parts < kLazyMaxParts ? parts : kLazyMaxParts;
-                split_slot[i] = slot;
+                split_slot[j] = row;
             }
         }
         const int32_t t0 = atomicAdd(&n_tasks, parts);
-        for (int32_t p = 0; p < parts; p++) L.task[t0 + p] = make_int4(u, p, parts, 0);
+        const int32_t k = place.x + 1;
+        for (int32_t p = 0; p < parts; p++) {
+            LazyTask t;
+            t.node = s;
+            t.row = row;
+            t.pos = place.x;
+            t.part = p;
+            t.k0 = k + int32_t(int64_t(desc) * p / parts);
+            t.k1 = k + int32_t(int64_t(desc) * (p + 1) / parts);
+            t.parts = parts;
+            t.pad = 0;
+            L.task[t0 + p] = t;
+        }
     }
     __syncthreads();
     // rows built in parts are ORed together by atomics: zero them first
@@ -1643,9 +1669,12 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
         uint32_t *row = L.rows + int64_t(split_slot[r]) * L.W;
         for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) row[i] = 0u;
     }
-    // 4. batch rows of missing nodes
-    for (int32_t b = threadIdx.x; b < B; b += blockDim.x)
-        if (L.slot_of[b] == kPending) L.slot_of[b] = L.miss_slot[vals[L.row_u[b]]];
+    // 3. every batch row's cache row
+#pragma unroll
+    for (int q = 0; q < kResolvePer; q++) {
+        const int32_t b = threadIdx.x + q * kResolveThreads;
+        if (b < B) L.slot_of[b] = at[q] >= 0 ? vals[at[q]] : slot[q];
+    }
     if (threadIdx.x == 0) {
         L.ctrl->n_miss = n_u;
         L.ctrl->n_tasks = n_tasks;
@@ -1677,26 +1706,34 @@ __device__ __forceinline__ uint64_t hash_pow(uint32_t j) {
 
 constexpr int kLazyNodesPerThread = 4;  // descendants resolved together by one thread
 
+// A task's row is a chain of loads: task, records, slot pair, payload, token
+// bytes (12 us of a step at K = 10,000, B = 256 with the node's place looked up
+// again and the token's id, length and bytes one after the other, 7.8-9.4 us
+// so). The moves it found are kept until the row is stored: inserted as they
+// are found, each one's compare-and-swap in the transition table held up the
+// row. (Moves beyond the list are inserted at once.)
+constexpr int kLazyMoves = 256;
+
 __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, PatchArgs a) {
     extern __shared__ uint32_t bits[];
+    __shared__ int2 moves[kLazyMoves];  // {token, end node}
+    __shared__ int32_t n_moves;
     pdl_launch_dependents();
+    for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) bits[i] = 0u;
+    if (threadIdx.x == 0) n_moves = 0;
     pdl_wait();  // the resolve's task list
     const int32_t n_tasks = __ldcg(&L.ctrl->n_tasks);
     const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(a.ht_key);
+    const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
     for (int32_t ti = blockIdx.x; ti < n_tasks; ti += gridDim.x) {
-        const int4 tk = __ldcg(L.task + ti);  // {miss, part, parts, -}
-        const int32_t s = L.miss_node[tk.x];
-        for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) bits[i] = 0u;
-        __syncthreads();
-        if (threadIdx.x == 0 && tk.y == 0 && __ldg(a.terminal + s)) atomicOr(bits + (a.eos >> 5), 1u << (a.eos & 31));
-        const int32_t pos = __ldg(L.pos_of + s);
-        const int32_t desc = __ldg(L.pre_size + pos) - 1;
-        const int32_t k0 = pos + 1 + int32_t(int64_t(desc) * tk.y / tk.z);
-        const int32_t k1 = pos + 1 + int32_t(int64_t(desc) * (tk.y + 1) / tk.z);
-        const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
+        const int4 t0 = __ldcg(reinterpret_cast<const int4 *>(L.task + ti));
+        const int4 t1 = __ldcg(reinterpret_cast<const int4 *>(L.task + ti) + 1);
+        const int32_t s = t0.x, slot_row = t0.y, pos = t0.z, part = t0.w, k0 = t1.x, k1 = t1.y, parts = t1.z;
         const ulonglong2 sh0 = __ldg(rec + 2 * int64_t(pos));
         const uint64_t ps = sh0.x;
         const int32_t d0 = int32_t(uint32_t(sh0.y));
+        __syncthreads();  // bits and n_moves are zero
+        if (threadIdx.x == 0 && part == 0 && __ldg(a.terminal + s)) atomicOr(bits + (a.eos >> 5), 1u << (a.eos & 31));
         for (int32_t kb = k0 + int32_t(threadIdx.x); kb < k1; kb += kLazyNodesPerThread * blockDim.x) {
             int32_t d[kLazyNodesPerThread], j[kLazyNodesPerThread];
             uint64_t pd[kLazyNodesPerThread];
@@ -1750,51 +1787,68 @@ __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, Pa
                     }
                 }
             }
+            // the matches' tokens: with the per-slot payload one load gives the
+            // id, length, offset and first 8 bytes, and only longer tokens read on
             int32_t tid[kLazyNodesPerThread];
-#pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++) tid[g] = slot[g] >= 0 ? __ldg(a.ht_val + slot[g]) : -1;
             int32_t tlen[kLazyNodesPerThread];
             uint32_t toff[kLazyNodesPerThread];
-#pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++) {
-                tlen[g] = tid[g] >= 0 ? int32_t(__ldg(a.tok_len + tid[g])) : -1;
-                toff[g] = tid[g] >= 0 ? __ldg(a.tok_off + tid[g]) : 0u;
-            }
             uint4 tb[kLazyNodesPerThread];
+            if (a.ht_pay) {
 #pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++)
-                tb[g] = tlen[g] == j[g] ? __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]))
-                                        : make_uint4(0u, 0u, 0u, 0u);
+                for (int g = 0; g < kLazyNodesPerThread; g++) {
+                    const uint4 p = slot[g] >= 0 ? __ldg(a.ht_pay + slot[g]) : make_uint4(0u, 0u, 0u, 0u);
+                    tid[g] = slot[g] >= 0 ? int32_t(p.x) : -1;
+                    tlen[g] = slot[g] >= 0 ? int32_t(p.y >> 27) : -1;
+                    toff[g] = (p.y & 0x07FFFFFFu) << 4;
+                    tb[g] = make_uint4(p.z, p.w, 0u, 0u);
+                }
+#pragma unroll
+                for (int g = 0; g < kLazyNodesPerThread; g++)
+                    if (j[g] > 8 && tlen[g] == j[g]) tb[g] = __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]));
+            } else {
+#pragma unroll
+                for (int g = 0; g < kLazyNodesPerThread; g++) tid[g] = slot[g] >= 0 ? __ldg(a.ht_val + slot[g]) : -1;
+#pragma unroll
+                for (int g = 0; g < kLazyNodesPerThread; g++) {
+                    tlen[g] = tid[g] >= 0 ? int32_t(__ldg(a.tok_len + tid[g])) : -1;
+                    toff[g] = tid[g] >= 0 ? __ldg(a.tok_off + tid[g]) : 0u;
+                }
+#pragma unroll
+                for (int g = 0; g < kLazyNodesPerThread; g++)
+                    tb[g] = tlen[g] == j[g] ? __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]))
+                                            : make_uint4(0u, 0u, 0u, 0u);
+            }
 #pragma unroll
             for (int g = 0; g < kLazyNodesPerThread; g++) {
                 // token t moves s to d: its bit, and the move for later advances
                 auto hit = [&](int32_t t) {
                     atomicOr(bits + (t >> 5), 1u << (t & 31));
-                    if (a.trans_fill) trans_insert(a.trans, a.trans_mask, s, t, d[g]);
+                    if (!a.trans_fill) return;
+                    const int32_t i = atomicAdd(&n_moves, 1);
+                    if (i < kLazyMoves) moves[i] = make_int2(t, d[g]);
+                    else trans_insert(a.trans, a.trans_mask, s, t, d[g]);
                 };
                 if (slow & (1u << g)) {
                     if (j[g] > kMaxClimb) probe(a, key[g], j[g], nullptr, d[g], hit);
                     else probe(a, key[g], j[g], &lab[g], d[g], hit);
                 } else if (tid[g] >= 0 && tlen[g] == j[g]) {
-                    // token byte i must equal the label j-1-i levels above d
-                    const uint32_t tw[4] = {tb[g].x, tb[g].y, tb[g].z, tb[g].w};
-                    bool eq = true;
-#pragma unroll
-                    for (int i = 0; i < kMaxClimb; i++)
-                        if (i < j[g]) eq = eq && byte_at(tw, i) == byte_at(lab[g], j[g] - 1 - i);
-                    if (eq) hit(tid[g]);
+                    if (spells_window(lab[g], tb[g], j[g])) hit(tid[g]);
                 }
             }
         }
         __syncthreads();
-        uint32_t *row = L.rows + int64_t(L.miss_slot[tk.x]) * L.W;
-        if (tk.z == 1) {
-            for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) row[i] = bits[i];
-        } else {
-            for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x)
-                if (bits[i]) atomicOr(row + i, bits[i]);
+        uint32_t *row = L.rows + int64_t(slot_row) * L.W;
+        const int32_t kept = n_moves < kLazyMoves ? n_moves : kLazyMoves;
+        for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) {
+            const uint32_t w = bits[i];
+            if (parts == 1) row[i] = w;
+            else if (w) atomicOr(row + i, w);
+            bits[i] = 0u;  // for the CTA's next task
         }
-        __syncthreads();  // bits are reused by the next task
+        for (int32_t i = threadIdx.x; i < kept; i += blockDim.x)
+            trans_insert(a.trans, a.trans_mask, s, moves[i].x, moves[i].y);
+        __syncthreads();  // moves are reused by the next task
+        if (threadIdx.x == 0) n_moves = 0;
     }
 }
 
@@ -1814,18 +1868,18 @@ __global__ void __launch_bounds__(kApplyThreads) k_lazy_gather(const uint32_t *_
 }
 
 // The pre-order records of the lazy rows: for position k, node d =
-// pre_node[k], pos_of[d] = k, d's depth and label window, and the path hash
+// pre_node[k], place[d] = {k, subtree size}, d's depth and label window, and the path hash
 // of d: the Horner polynomial of the token table's hash over (label + 1) of
 // the edges from the root to d, P(d) = P(parent) * B + label(d) + 1
 // (mod 2^64), summed here by climbing to the root. The path from s down to a
 // descendant d, j edges long, then hashes to P(d) - P(s) * B^j.
 __global__ void k_lazy_tables(const int32_t *__restrict__ pre_node, const int32_t *__restrict__ pre_depth,
                               const int32_t *__restrict__ parent, const uint8_t *__restrict__ label,
-                              const ulonglong2 *__restrict__ window, int32_t n, int32_t *__restrict__ pos_of,
-                              LazyNode *__restrict__ pre) {
+                              const int32_t *__restrict__ pre_size, const ulonglong2 *__restrict__ window,
+                              int32_t n, int2 *__restrict__ place, LazyNode *__restrict__ pre) {
     for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int32_t d = pre_node[k];
-        pos_of[d] = k;
+        place[d] = make_int2(k, pre_size[k]);
         uint64_t h = 0, pw = 1;
         for (int32_t y = d; __ldg(parent + y) >= 0; y = __ldg(parent + y)) {
             h += (uint64_t(__ldg(label + y)) + 1ull) * pw;
@@ -2210,8 +2264,8 @@ cudaError_t launch_lazy_tables(const DevTrie &t, const DevLazy &L, int32_t n_nod
         return e;
     if (n_nodes <= 0) return cudaSuccess;
     const int grid = grid_for(n_nodes, 256, 4096);
-    k_lazy_tables<<<grid, 256, 0, st>>>(L.pre_node, L.pre_depth, t.parent, t.label, t.window, n_nodes, L.pos_of,
-                                        L.pre);
+    k_lazy_tables<<<grid, 256, 0, st>>>(L.pre_node, L.pre_depth, t.parent, t.label, L.pre_size, t.window, n_nodes,
+                                        L.place, L.pre);
     return cudaGetLastError();
 }
 
@@ -2226,14 +2280,8 @@ cudaError_t launch_lazy(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bo
     la.stamp = L.stamp;
     la.ctrl = L.ctrl;
     la.slot_of = L.slot_of;
-    la.miss_node = L.miss_node;
-    la.miss_slot = L.miss_slot;
-    la.row_u = L.row_u;
     la.task = L.task;
-    la.pre_node = L.pre_node;
-    la.pre_depth = L.pre_depth;
-    la.pre_size = L.pre_size;
-    la.pos_of = L.pos_of;
+    la.place = L.place;
     la.pre = L.pre;
     la.C = L.C;
     la.n_sets = L.C / kLazyWays;

@@ -312,6 +312,20 @@ struct LazyCtrl {
     unsigned long long misses;      // batch rows whose node row was computed
 };
 
+// What one CTA of the row kernel does: the row of `node` (at pre-order
+// position pos), or one part of it, from the positions k0 .. k1 - 1 of its
+// subtree.
+struct alignas(16) LazyTask {
+    int32_t node;
+    int32_t row;
+    int32_t pos;
+    int32_t part;
+    int32_t k0;
+    int32_t k1;
+    int32_t parts;
+    int32_t pad;
+};
+
 // One node of the depth-first pre-order, as the lazy-row kernel reads it (a
 // subtree is a contiguous run of these, 32 bytes each).
 struct LazyNode {
@@ -334,14 +348,11 @@ struct DevLazy {
     uint32_t *stamp = nullptr;      // [C] call that last used the row (0 never)
     LazyCtrl *ctrl = nullptr;
     int32_t *slot_of = nullptr;     // [max_batch] row of each batch row, < 0: {EOS}
-    int32_t *miss_node = nullptr;   // [max_batch] nodes whose rows the call computes
-    int32_t *miss_slot = nullptr;   // [max_batch] where
-    int32_t *row_u = nullptr;       // [max_batch] scratch
-    int4 *task = nullptr;           // [max_batch + kLazySplitRows * kLazyMaxParts] {miss, part, parts, -}
+    LazyTask *task = nullptr;       // [max_batch + kLazySplitRows * kLazyMaxParts]
     int32_t *pre_node = nullptr;    // [n] pre-order tables of the trie (HostTrie)
     int32_t *pre_depth = nullptr;   // [n]
     int32_t *pre_size = nullptr;    // [n]
-    int32_t *pos_of = nullptr;      // [n] pre-order position of each node
+    int2 *place = nullptr;          // [n] pre-order position and subtree size of each node
     LazyNode *pre = nullptr;        // [n] by pre-order position
 };
 
@@ -490,7 +501,7 @@ cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab
                                int num_sms, cudaStream_t st);
 cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
                                int num_sms, cudaStream_t st);
-// Lazy rows: pos_of from the pre-order tables and the path hashes (once, at set-up).
+// Lazy rows: place from the pre-order tables and the path hashes (once, at set-up).
 cudaError_t launch_lazy_tables(const DevTrie &t, const DevLazy &L, int32_t n_nodes, cudaStream_t st);
 // One lazy call: map the batch's states (after the advance when tokens is not
 // null) to cache rows, compute the missing rows, then apply them to the
