@@ -1704,8 +1704,6 @@ __device__ __forceinline__ uint64_t hash_pow(uint32_t j) {
     return r;
 }
 
-constexpr int kLazyNodesPerThread = 4;  // descendants resolved together by one thread
-
 // A task's row is a chain of loads: task, records, slot pair, payload, token
 // bytes (12 us of a step at K = 10,000, B = 256 with the node's place looked up
 // again and the token's id, length and bytes one after the other, 7.8-9.4 us
@@ -1713,6 +1711,123 @@ constexpr int kLazyNodesPerThread = 4;  // descendants resolved together by one 
 // are found, each one's compare-and-swap in the transition table held up the
 // row. (Moves beyond the list are inserted at once.)
 constexpr int kLazyMoves = 256;
+
+// The tokens on the paths from s (at depth d0, path hash ps) down to the
+// descendants at pre-order positions k0 .. k1 - 1: their bits, and the moves
+// they make. G descendants of a thread are resolved together, each round of
+// loads issued for all of them; with at most one a thread G = 1, because empty
+// ones cost their instructions all the same (four a thread for every subtree:
+// 24.7 us a step at K = 10,000, B = 256, 24.3 us so; K = 100, B = 1 9.4 and 8.8
+// us).
+template <int G>
+__device__ __forceinline__ void search_descendants(const LazyArgs &L, const PatchArgs &a, int32_t s, uint64_t ps,
+                                                   int32_t d0, int32_t k0, int32_t k1, uint32_t *bits, int2 *moves,
+                                                   int32_t *n_moves) {
+    const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(a.ht_key);
+    const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
+    for (int32_t kb = k0 + int32_t(threadIdx.x); kb < k1; kb += G * blockDim.x) {
+        int32_t d[G], j[G];
+        uint64_t pd[G];
+        uint32_t lab[G][4];
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            const int32_t k = kb + g * int32_t(blockDim.x);
+            ulonglong2 r0 = make_ulonglong2(0ull, 0ull), r1 = make_ulonglong2(0ull, 0ull);
+            if (k < k1) {
+                r0 = __ldg(rec + 2 * int64_t(k));
+                r1 = __ldg(rec + 2 * int64_t(k) + 1);
+            }
+            pd[g] = r0.x;
+            j[g] = k < k1 ? int32_t(uint32_t(r0.y)) - d0 : 0;
+            d[g] = int32_t(uint32_t(r0.y >> 32));
+            if (j[g] > a.lmax) j[g] = 0;  // no token is this long
+            lab[g][0] = uint32_t(r1.x);
+            lab[g][1] = uint32_t(r1.x >> 32);
+            lab[g][2] = uint32_t(r1.y);
+            lab[g][3] = uint32_t(r1.y >> 32);
+        }
+        uint64_t key[G];
+        ulonglong2 f[G];
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            key[g] = hash_finish(pd[g] - ps * hash_pow(uint32_t(j[g])), uint32_t(j[g]));
+            f[g] = j[g] > 0 ? __ldg(pairs + (uint32_t(key[g] >> 1) & a.pairs_mask)) : make_ulonglong2(0ull, 0ull);
+        }
+        // keys are resolved together (find_slots); paths longer than the
+        // label window, and full first pairs in a vocabulary where tokens
+        // share keys, take the sequential probe
+        int32_t slot[G];
+        uint32_t slow = 0;
+        if (!a.dup_keys) {
+            uint32_t pending = 0;
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                if (j[g] > kMaxClimb) slow |= 1u << g;
+                else if (j[g] > 0) pending |= 1u << g;
+            }
+            find_slots<G>(a, key, pending, f, slot);
+        } else {
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                const bool m0 = f[g].x == key[g], m1 = f[g].y == key[g];
+                const uint32_t pr = uint32_t(key[g] >> 1) & a.pairs_mask;
+                slot[g] = -1;
+                if (j[g] > 0) {
+                    if (j[g] > kMaxClimb || f[g].y != 0ull) slow |= 1u << g;
+                    else if (m0 || m1) slot[g] = int32_t(2 * pr + (m0 ? 0 : 1));
+                }
+            }
+        }
+        // the matches' tokens: with the per-slot payload one load gives the
+        // id, length, offset and first 8 bytes, and only longer tokens read on
+        int32_t tid[G];
+        int32_t tlen[G];
+        uint32_t toff[G];
+        uint4 tb[G];
+        if (a.ht_pay) {
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                const uint4 p = slot[g] >= 0 ? __ldg(a.ht_pay + slot[g]) : make_uint4(0u, 0u, 0u, 0u);
+                tid[g] = slot[g] >= 0 ? int32_t(p.x) : -1;
+                tlen[g] = slot[g] >= 0 ? int32_t(p.y >> 27) : -1;
+                toff[g] = (p.y & 0x07FFFFFFu) << 4;
+                tb[g] = make_uint4(p.z, p.w, 0u, 0u);
+            }
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                if (j[g] > 8 && tlen[g] == j[g]) tb[g] = __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]));
+        } else {
+#pragma unroll
+            for (int g = 0; g < G; g++) tid[g] = slot[g] >= 0 ? __ldg(a.ht_val + slot[g]) : -1;
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                tlen[g] = tid[g] >= 0 ? int32_t(__ldg(a.tok_len + tid[g])) : -1;
+                toff[g] = tid[g] >= 0 ? __ldg(a.tok_off + tid[g]) : 0u;
+            }
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                tb[g] = tlen[g] == j[g] ? __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]))
+                                        : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            // token t moves s to d: its bit, and the move for later advances
+            auto hit = [&](int32_t t) {
+                atomicOr(bits + (t >> 5), 1u << (t & 31));
+                if (!a.trans_fill) return;
+                const int32_t i = atomicAdd(n_moves, 1);
+                if (i < kLazyMoves) moves[i] = make_int2(t, d[g]);
+                else trans_insert(a.trans, a.trans_mask, s, t, d[g]);
+            };
+            if (slow & (1u << g)) {
+                if (j[g] > kMaxClimb) probe(a, key[g], j[g], nullptr, d[g], hit);
+                else probe(a, key[g], j[g], &lab[g], d[g], hit);
+            } else if (tid[g] >= 0 && tlen[g] == j[g]) {
+                if (spells_window(lab[g], tb[g], j[g])) hit(tid[g]);
+            }
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, PatchArgs a) {
     extern __shared__ uint32_t bits[];
@@ -1723,7 +1838,6 @@ __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, Pa
     if (threadIdx.x == 0) n_moves = 0;
     pdl_wait();  // the resolve's task list
     const int32_t n_tasks = __ldcg(&L.ctrl->n_tasks);
-    const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(a.ht_key);
     const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
     for (int32_t ti = blockIdx.x; ti < n_tasks; ti += gridDim.x) {
         const int4 t0 = __ldcg(reinterpret_cast<const int4 *>(L.task + ti));
@@ -1734,108 +1848,8 @@ __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, Pa
         const int32_t d0 = int32_t(uint32_t(sh0.y));
         __syncthreads();  // bits and n_moves are zero
         if (threadIdx.x == 0 && part == 0 && __ldg(a.terminal + s)) atomicOr(bits + (a.eos >> 5), 1u << (a.eos & 31));
-        for (int32_t kb = k0 + int32_t(threadIdx.x); kb < k1; kb += kLazyNodesPerThread * blockDim.x) {
-            int32_t d[kLazyNodesPerThread], j[kLazyNodesPerThread];
-            uint64_t pd[kLazyNodesPerThread];
-            uint32_t lab[kLazyNodesPerThread][4];
-#pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++) {
-                const int32_t k = kb + g * int32_t(blockDim.x);
-                ulonglong2 r0 = make_ulonglong2(0ull, 0ull), r1 = make_ulonglong2(0ull, 0ull);
-                if (k < k1) {
-                    r0 = __ldg(rec + 2 * int64_t(k));
-                    r1 = __ldg(rec + 2 * int64_t(k) + 1);
-                }
-                pd[g] = r0.x;
-                j[g] = k < k1 ? int32_t(uint32_t(r0.y)) - d0 : 0;
-                d[g] = int32_t(uint32_t(r0.y >> 32));
-                if (j[g] > a.lmax) j[g] = 0;  // no token is this long
-                lab[g][0] = uint32_t(r1.x);
-                lab[g][1] = uint32_t(r1.x >> 32);
-                lab[g][2] = uint32_t(r1.y);
-                lab[g][3] = uint32_t(r1.y >> 32);
-            }
-            uint64_t key[kLazyNodesPerThread];
-            ulonglong2 f[kLazyNodesPerThread];
-#pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++) {
-                key[g] = hash_finish(pd[g] - ps * hash_pow(uint32_t(j[g])), uint32_t(j[g]));
-                f[g] = j[g] > 0 ? __ldg(pairs + (uint32_t(key[g] >> 1) & a.pairs_mask)) : make_ulonglong2(0ull, 0ull);
-            }
-            // keys are resolved together (find_slots); paths longer than the
-            // label window, and full first pairs in a vocabulary where tokens
-            // share keys, take the sequential probe
-            int32_t slot[kLazyNodesPerThread];
-            uint32_t slow = 0;
-            if (!a.dup_keys) {
-                uint32_t pending = 0;
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++) {
-                    if (j[g] > kMaxClimb) slow |= 1u << g;
-                    else if (j[g] > 0) pending |= 1u << g;
-                }
-                find_slots<kLazyNodesPerThread>(a, key, pending, f, slot);
-            } else {
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++) {
-                    const bool m0 = f[g].x == key[g], m1 = f[g].y == key[g];
-                    const uint32_t pr = uint32_t(key[g] >> 1) & a.pairs_mask;
-                    slot[g] = -1;
-                    if (j[g] > 0) {
-                        if (j[g] > kMaxClimb || f[g].y != 0ull) slow |= 1u << g;
-                        else if (m0 || m1) slot[g] = int32_t(2 * pr + (m0 ? 0 : 1));
-                    }
-                }
-            }
-            // the matches' tokens: with the per-slot payload one load gives the
-            // id, length, offset and first 8 bytes, and only longer tokens read on
-            int32_t tid[kLazyNodesPerThread];
-            int32_t tlen[kLazyNodesPerThread];
-            uint32_t toff[kLazyNodesPerThread];
-            uint4 tb[kLazyNodesPerThread];
-            if (a.ht_pay) {
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++) {
-                    const uint4 p = slot[g] >= 0 ? __ldg(a.ht_pay + slot[g]) : make_uint4(0u, 0u, 0u, 0u);
-                    tid[g] = slot[g] >= 0 ? int32_t(p.x) : -1;
-                    tlen[g] = slot[g] >= 0 ? int32_t(p.y >> 27) : -1;
-                    toff[g] = (p.y & 0x07FFFFFFu) << 4;
-                    tb[g] = make_uint4(p.z, p.w, 0u, 0u);
-                }
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++)
-                    if (j[g] > 8 && tlen[g] == j[g]) tb[g] = __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]));
-            } else {
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++) tid[g] = slot[g] >= 0 ? __ldg(a.ht_val + slot[g]) : -1;
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++) {
-                    tlen[g] = tid[g] >= 0 ? int32_t(__ldg(a.tok_len + tid[g])) : -1;
-                    toff[g] = tid[g] >= 0 ? __ldg(a.tok_off + tid[g]) : 0u;
-                }
-#pragma unroll
-                for (int g = 0; g < kLazyNodesPerThread; g++)
-                    tb[g] = tlen[g] == j[g] ? __ldg(reinterpret_cast<const uint4 *>(a.blob + toff[g]))
-                                            : make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int g = 0; g < kLazyNodesPerThread; g++) {
-                // token t moves s to d: its bit, and the move for later advances
-                auto hit = [&](int32_t t) {
-                    atomicOr(bits + (t >> 5), 1u << (t & 31));
-                    if (!a.trans_fill) return;
-                    const int32_t i = atomicAdd(&n_moves, 1);
-                    if (i < kLazyMoves) moves[i] = make_int2(t, d[g]);
-                    else trans_insert(a.trans, a.trans_mask, s, t, d[g]);
-                };
-                if (slow & (1u << g)) {
-                    if (j[g] > kMaxClimb) probe(a, key[g], j[g], nullptr, d[g], hit);
-                    else probe(a, key[g], j[g], &lab[g], d[g], hit);
-                } else if (tid[g] >= 0 && tlen[g] == j[g]) {
-                    if (spells_window(lab[g], tb[g], j[g])) hit(tid[g]);
-                }
-            }
-        }
+        if (k1 - k0 <= kLazyRowThreads) search_descendants<1>(L, a, s, ps, d0, k0, k1, bits, moves, &n_moves);
+        else search_descendants<4>(L, a, s, ps, d0, k0, k1, bits, moves, &n_moves);
         __syncthreads();
         uint32_t *row = L.rows + int64_t(slot_row) * L.W;
         const int32_t kept = n_moves < kLazyMoves ? n_moves : kLazyMoves;

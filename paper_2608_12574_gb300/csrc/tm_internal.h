@@ -297,11 +297,14 @@ constexpr int32_t kLazyMaxCacheRows = int32_t(1) << 30;  // cache rows + call ro
 constexpr int64_t kLazyMaxWords = 16384;  // row built in shared memory (64 KB): V <= 524,288
 // A missing row whose subtree has more than kLazyPartNodes nodes is computed
 // in parts by several CTAs (at most kLazyMaxParts per row), for at most
-// kLazySplitRows rows per call (splitting only pays while few rows are
-// missing; with many the grid is full anyway).
+// kLazySplitRows rows per call: a subtree left whole is one CTA's, and a step
+// of K = 74,719, V = 262,144, B = 256 without a cache, whose 26 letters hold
+// 4,300 nodes each, took 70.5 us with 16 rows, 67.4 with 32, 65.1 with 64, 65.6
+// with 128 (parts of 512, 1,536 and 2,048 nodes with 64 rows: 70.5, 66.3 and
+// 66.4 us; K = 10,000 24.3 us with 1,024, 25.1-25.5 us with the others).
 constexpr int32_t kLazyPartNodes = 1024;
 constexpr int32_t kLazyMaxParts = 64;
-constexpr int32_t kLazySplitRows = 16;
+constexpr int32_t kLazySplitRows = 64;
 
 struct LazyCtrl {
     uint32_t now;                   // call counter (stamps of rows used by this call)
