@@ -1055,14 +1055,14 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
     // token buffer is sized by it and nothing is read back; otherwise the
     // exact total is read back between the two walks (host-synchronous).
     const int64_t bound = int64_t(n) * (int64_t(lmax) * voc->rt_mult + 1);
-    const bool by_bound = bound <= std::max<int64_t>(kListBoundEntries, L.tok_cap);
+    const bool by_bound = bound <= std::max<int64_t>(kListBoundEntries, L.cap);
     if (!L.base) {  // per-row counts, offsets, scan scratch (and a first token buffer, in one block)
         Layout lay;
         const size_t o_cnt = lay.add(sizeof(int32_t) * size_t(n));
         const size_t o_off = lay.add(sizeof(int64_t) * (size_t(n) + 1));
         const size_t o_tile = lay.add(sizeof(int64_t) * (size_t(n) / 4096 + 2));
         const size_t o_tot = lay.add(sizeof(int64_t));
-        const size_t o_tok = by_bound ? lay.add(2 * sizeof(int32_t) * size_t(std::max<int64_t>(bound, 1))) : 0;
+        const size_t o_tok = by_bound ? lay.add(sizeof(int2) * size_t(std::max<int64_t>(bound, 1))) : 0;
         void *base = take_spare_block(dev, lay.total);
         if (!base && (rc = pool_alloc(dev, lay.total, stream, &base, "the valid lists")) != TRIE_OK) return rc;
         cudaEvent_t done = nullptr;
@@ -1080,27 +1080,24 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
         L.tile_sum = reinterpret_cast<int64_t *>(b + o_tile);
         L.total = reinterpret_cast<int64_t *>(b + o_tot);
         if (by_bound) {
-            L.toks = reinterpret_cast<int32_t *>(b + o_tok);
-            L.tok_cap = std::max<int64_t>(bound, 1);
-            L.ends = L.toks + L.tok_cap;
-            L.toks_separate = false;
+            L.entries = reinterpret_cast<int2 *>(b + o_tok);
+            L.cap = std::max<int64_t>(bound, 1);
+            L.entries_separate = false;
         }
     }
     const int sms = num_sms(dev);
     auto grow = [&](int64_t need) -> int {
-        if (need <= L.tok_cap) return TRIE_OK;
-        if (L.toks_separate) pool_free(L.toks);  // earlier apply calls may still read it
-        L.toks = nullptr;                         // (a buffer inside the block at base stays there)
-        L.ends = nullptr;
-        L.tok_cap = 0;
-        void *toks = nullptr;
+        if (need <= L.cap) return TRIE_OK;
+        if (L.entries_separate) pool_free(L.entries);  // earlier apply calls may still read it
+        L.entries = nullptr;                            // (a buffer inside the block at base stays there)
+        L.cap = 0;
+        void *p = nullptr;
         need = std::max<int64_t>(need, 1);
-        int r = pool_alloc(dev, 2 * sizeof(int32_t) * size_t(need), stream, &toks, "the valid-list tokens");
+        int r = pool_alloc(dev, sizeof(int2) * size_t(need), stream, &p, "the valid-list entries");
         if (r != TRIE_OK) return r;
-        L.toks = static_cast<int32_t *>(toks);
-        L.ends = L.toks + need;
-        L.tok_cap = need;
-        L.toks_separate = true;
+        L.entries = static_cast<int2 *>(p);
+        L.cap = need;
+        L.entries_separate = true;
         return TRIE_OK;
     };
     auto failed = [&](int r) {
@@ -1198,8 +1195,17 @@ int trie_copy_lists(trie_t h, int64_t *d_offsets, int32_t *d_tokens, cudaStream_
         if (e != cudaSuccess) return fail_cuda(e, "copying the list offsets");
     }
     if (d_tokens && L.n_valid > 0) {
-        cudaError_t e = cudaMemcpyAsync(d_tokens, L.toks, sizeof(int32_t) * size_t(L.n_valid),
-                                        cudaMemcpyDeviceToDevice, stream);
+        // the tokens out of the {token, end node} entries: by a kernel into the
+        // handle's device, by a strided copy into any other memory
+        DeviceGuard g(h->dev.device);
+        cudaPointerAttributes at = {};
+        const bool here = cudaPointerGetAttributes(&at, d_tokens) == cudaSuccess &&
+                          at.type == cudaMemoryTypeDevice && at.device == h->dev.device &&
+                          (reinterpret_cast<uintptr_t>(d_tokens) & 3u) == 0;
+        cudaGetLastError();
+        cudaError_t e = here ? tmk::launch_copy_tokens(L, L.n_valid, d_tokens, num_sms(h->dev.device), stream)
+                             : cudaMemcpy2DAsync(d_tokens, sizeof(int32_t), L.entries, sizeof(int2), sizeof(int32_t),
+                                                 size_t(L.n_valid), cudaMemcpyDeviceToDevice, stream);
         if (e != cudaSuccess) return fail_cuda(e, "copying the list tokens");
     }
     return TRIE_OK;
@@ -1503,7 +1509,7 @@ int trie_destroy(trie_t h) {
     if (h->dev.base || h->lists.base) {
         DeviceGuard g(h->dev.device);
         // after the work on the device that may still read these
-        if (h->lists.toks_separate) pool_free(h->lists.toks);
+        if (h->lists.entries_separate) pool_free(h->lists.entries);
         if (h->lists.base) {
             cudaDeviceSynchronize();  // no queued work still uses the block
             give_spare_block(h->dev.device, h->lists.base, h->lists.base_bytes, nullptr, 0);
@@ -1568,14 +1574,14 @@ int trie_destroy_async(trie_t h, cudaStream_t stream) {
     // reference frees device memory, which a stream callback must not do)
     std::shared_ptr<tmk::DevVocab> v1 = std::move(h->vocab), v2 = std::move(h->trans_vocab),
                                    v3 = std::move(h->lazy.vocab);
-    int dev = h->dev.base || h->lists.base || h->lists.toks ? h->dev.device : h->lazy.device;
+    int dev = h->dev.base || h->lists.base || h->lists.entries ? h->dev.device : h->lazy.device;
     if (h->lazy.base) {
         DeviceGuard g(h->lazy.device);
         free_on(h->lazy.base);
     }
-    if (h->dev.base || h->lists.base || h->lists.toks) {
+    if (h->dev.base || h->lists.base || h->lists.entries) {
         DeviceGuard g(h->dev.device);
-        if (h->lists.toks_separate) free_on(h->lists.toks);
+        if (h->lists.entries_separate) free_on(h->lists.entries);
         if (h->lists.base) {  // kept for a later handle once the queued work is done
             cudaEvent_t ev = nullptr;
             if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&

@@ -1238,11 +1238,18 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_rows(const int32_t *__res
     for (int j = 0; j < kScanPer; j++) v += c[j];
     int64_t total;
     int64_t run = tile_off[blockIdx.x] + block_exclusive_scan(v, sw, &total);
+    // through shared memory, so that a warp stores 256 contiguous bytes (each
+    // thread storing its own four offsets: 20 us on the 4.77 M-node forest, 11
+    // us so)
+    __shared__ int64_t out[kScanTile];
 #pragma unroll
     for (int j = 0; j < kScanPer; j++) {
-        if (base + j < n) off[base + j + 1] = run;
+        out[threadIdx.x * kScanPer + j] = run;
         run += c[j];
     }
+    __syncthreads();
+    const int64_t first = int64_t(blockIdx.x) * kScanTile;
+    for (int i = threadIdx.x; i < kScanTile && first + i < n; i += kScanThreads) off[first + i + 1] = out[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) off[0] = 0;
 }
 
@@ -1259,6 +1266,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_rows(const int32_t *__res
 // writes them at positions claimed from the rows' offsets (order within a row
 // unspecified).
 
+// An entry's token and the node it leads to are stored together: bound by the
+// number of its scattered operations, the writing walk of the 4.77 M-node
+// forest took 139 us with two arrays, 135 us so (stored a step later, under the
+// next look-up, 144 us).
 struct WalkArgs {
     const uint8_t *terminal;
     const int32_t *parent;
@@ -1271,9 +1282,8 @@ struct WalkArgs {
     const int32_t *tok_next;   // tokens with the same bytes, or null
     int32_t *count;            // [n] entries per row (counting walk)
     unsigned long long *off;   // [n + 1]: off[i + 1] = next position of row i (writing walk)
-    int32_t *toks;
-    int32_t *ends;             // [tok_cap]: the node each entry's token leads to (FINISHED for EOS)
-    unsigned long long tok_cap;  // entries toks holds (a write past it is dropped)
+    int2 *entries;             // [cap] {token, the node it leads to (FINISHED for EOS)}
+    unsigned long long cap;    // entries it holds (a write past it is dropped)
 };
 
 constexpr int kWalkThreads = 256;  // also the 256 root edges each CTA stages
@@ -1325,10 +1335,10 @@ __global__ void k_rt_insert(const int32_t *__restrict__ parent, const uint8_t *_
 // nodes' ancestors are neighbours, so these loads fall together and come from
 // L1 and L2, where reading each entry's row from the 64-byte ancestor rows of
 // the dense compile's tables was 305 MB of DRAM reads a walk on the 4.77 M-node
-// forest (count walk 132 us, 98 us so; write walk 177 and 139 us; and the
+// forest (count walk 132 us, 98 us so; write walk 177 and 135 us; and the
 // forest needs no such tables). Bound by the L1's look-ups of the random edge
-// slots (two, three or four nodes a lane, their loads side by side: 272, 381
-// and 376 us for both walks and the scan, 264 us with one). Called by whole warps, whose lanes stay
+// slots (two, three or four nodes a lane, their loads side by side: 8, 117 and
+// 112 us more for both walks together). Called by whole warps, whose lanes stay
 // together until the longest walk ends: with a return at each lane's own end
 // the lanes ran on one by one (326 and 520 us).
 template <typename Tok>
@@ -1387,10 +1397,7 @@ __global__ void __launch_bounds__(kWalkThreads) k_list_walk(WalkArgs a) {
     auto emit = [&](int32_t row, int32_t t, int32_t end) {
         if (kWrite) {
             const unsigned long long p = atomicAdd(a.off + row + 1, 1ull);
-            if (p < a.tok_cap) {
-                a.toks[p] = t;
-                a.ends[p] = end;
-            }
+            if (p < a.cap) a.entries[p] = make_int2(t, end);
         } else {
             atomicAdd(a.count + row, 1);
         }
@@ -1414,13 +1421,12 @@ __global__ void __launch_bounds__(kWalkThreads) k_list_walk(WalkArgs a) {
 template <int kElt, bool kAdvance>
 __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict__ logits,
                                                                const int64_t *__restrict__ off,
-                                                               const int32_t *__restrict__ toks, AdvanceArgs aa,
+                                                               const int2 *__restrict__ entries, AdvanceArgs aa,
                                                                const int32_t *__restrict__ states,
                                                                const int32_t *__restrict__ tokens,
                                                                int32_t *__restrict__ states_out,
                                                                int32_t *__restrict__ err, int32_t B, int32_t V,
-                                                               int32_t n_nodes, int32_t parts,
-                                                               const int32_t *__restrict__ ends) {
+                                                               int32_t n_nodes, int32_t parts) {
     constexpr int kSegChunks = 1024 / (16 / kElt);
     constexpr int kWords = 8 * 32;
     __shared__ __align__(128) uint4 tile[kSegChunks];
@@ -1441,14 +1447,13 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict_
         // from a node, the move is the entry of the token in the node's list
         // (its end node, FINISHED for EOS), DEAD if the token is not there:
         // the advance's rules, in two dependent loads instead of a byte walk
-        // (each entry's token and end are loaded together)
         const int32_t t = __ldg(tokens + b);
-        const bool listed = ends && s0 >= 0 && s0 < n_nodes && t >= 0 && t < V;
+        const bool listed = s0 >= 0 && s0 < n_nodes && t >= 0 && t < V;
         if (listed) {
             const int64_t lo = __ldg(off + s0), hi = __ldg(off + s0 + 1);
             for (int64_t i = lo + threadIdx.x; i < hi; i += kApplyThreads) {
-                const int32_t tk = __ldg(toks + i), en = __ldg(ends + i);
-                if (tk == t) moved = en;
+                const int2 e = __ldg(entries + i);
+                if (e.x == t) moved = e.y;
             }
         }
         __syncthreads();
@@ -1473,7 +1478,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict_
     };
     if (s >= 0 && s < n_nodes) {
         const int64_t lo = __ldg(off + s), hi = __ldg(off + s + 1);
-        for (int64_t i = lo + threadIdx.x; i < hi; i += kApplyThreads) set_bit(__ldg(toks + i));
+        for (int64_t i = lo + threadIdx.x; i < hi; i += kApplyThreads) set_bit(__ldg(entries + i).x);
     } else if (threadIdx.x == 0) {
         set_bit(eos);  // FINISHED, DEAD, not a node: {EOS}
     }
@@ -2195,9 +2200,8 @@ WalkArgs walk_args(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const D
     a.tok_next = v.tok_next;
     a.count = L.count;
     a.off = reinterpret_cast<unsigned long long *>(L.off);
-    a.toks = L.toks;
-    a.ends = L.ends;
-    a.tok_cap = static_cast<unsigned long long>(L.tok_cap);
+    a.entries = L.entries;
+    a.cap = static_cast<unsigned long long>(L.cap);
     return a;
 }
 
@@ -2222,6 +2226,22 @@ cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab
     return cudaSuccess;
 }
 
+namespace {
+
+__global__ void k_copy_tokens(const int2 *__restrict__ entries, int64_t n, int32_t *__restrict__ tokens) {
+    pdl_launch_dependents();
+    pdl_wait();  // the entries come from earlier kernels, and those may still read the destination
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+        tokens[i] = entries[i].x;
+}
+
+}  // namespace
+
+cudaError_t launch_copy_tokens(const DevLists &L, int64_t n, int32_t *tokens, int num_sms, cudaStream_t st) {
+    return launch_pdl(k_copy_tokens, grid_for(n, 256, int64_t(num_sms) * 8), 256, st,
+                      static_cast<const int2 *>(L.entries), n, tokens);
+}
+
 cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
                                int num_sms, cudaStream_t st) {
     const WalkArgs a = walk_args(t, n_nodes, v, L);
@@ -2237,13 +2257,13 @@ cudaError_t launch_lists(void *logits, int dtype, const DevLists &L, const Advan
     const int32_t parts = int32_t((int64_t(V) + 8191) / 8192);
     const int64_t grid = int64_t(B) * parts;
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    const int32_t *tk = L.toks;
+    const int2 *en = L.entries;
     const int64_t *of = L.off;
     const AdvanceArgs a = aa ? *aa : AdvanceArgs{};
     auto *kernel = dtype == 0 ? (aa ? k_apply_lists<4, true> : k_apply_lists<4, false>)
                               : (aa ? k_apply_lists<2, true> : k_apply_lists<2, false>);
-    return launch_pdl(kernel, grid, kApplyThreads, st, logits, of, tk, a, states, tokens, states_out, err, B, V,
-                      n_nodes, parts, L.ends);
+    return launch_pdl(kernel, grid, kApplyThreads, st, logits, of, en, a, states, tokens, states_out, err, B, V,
+                      n_nodes, parts);
 }
 
 }  // namespace

@@ -272,16 +272,15 @@ struct DevTrie {
 
 // Device storage of the sparse valid lists of a handle (library-owned).
 struct DevLists {
-    void *base = nullptr;           // count, off, tile_sum, total (and a first token buffer)
+    void *base = nullptr;           // count, off, tile_sum, total (and a first entry buffer)
     size_t base_bytes = 0;
     int32_t *count = nullptr;       // [n] entries per row (the counting walk)
     int64_t *off = nullptr;         // [n + 1]
     int64_t *tile_sum = nullptr;    // [tiles]
     int64_t *total = nullptr;       // [1]
-    int32_t *toks = nullptr;        // [tok_cap]: in the block at base, or a separate allocation
-    int32_t *ends = nullptr;        // [tok_cap] after toks: the node each entry's token leads to
-    int64_t tok_cap = 0;
-    bool toks_separate = false;     // toks (with ends) is an allocation of its own
+    int2 *entries = nullptr;        // [cap] {token, the node it leads to}: in the block at base, or its own allocation
+    int64_t cap = 0;
+    bool entries_separate = false;
     int64_t n_valid = -1;           // entries of the last build, -1 before any (read back on demand)
     bool n_valid_on_device = false; // n_valid is still only in *total
     cudaEvent_t done = nullptr;     // recorded after the last build's kernels
@@ -498,10 +497,12 @@ cudaError_t launch_rt_build(const int32_t *parent, const uint8_t *label, const i
 // zero the per-row counts, count every (row, token) entry, scan the counts
 // into L.off (shifted one place up: off[i + 1] = the first position of row
 // i) and *L.total. Write: walk again, writing every entry at the position
-// claimed from off[row + 1] into L.toks (entries past L.tok_cap are
+// claimed from off[row + 1] into L.entries (those past L.cap are
 // dropped); afterwards L.off holds the rows' offsets.
 cudaError_t launch_lists_count(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
                                int num_sms, cudaStream_t st);
+// The tokens of the first n entries.
+cudaError_t launch_copy_tokens(const DevLists &L, int64_t n, int32_t *tokens, int num_sms, cudaStream_t st);
 cudaError_t launch_lists_write(const DevTrie &t, int32_t n_nodes, const DevVocab &v, const DevLists &L,
                                int num_sms, cudaStream_t st);
 // Lazy rows: place from the pre-order tables and the path hashes (once, at set-up).

@@ -286,3 +286,20 @@ def test_lists_errors(cuda):
     assert T.trie_compile_lists(h, vb, vo, 4) == 4   # root: a, ab; 'a': b; 'ab': EOS
     with pytest.raises(T.TrieError):
         T.trie_apply_lists(h, torch.zeros((1, 5), device=cuda), torch.zeros(1, dtype=torch.int32, device=cuda))
+
+
+def test_copy_lists_into_host_memory(cuda):
+    """trie_copy_lists takes any memory a copy takes: pinned host tokens equal
+    the device copy's."""
+    import ctypes
+
+    import torch
+    strings, toks = random_case(77)
+    h = T.trie_build(*W.pack(strings))
+    T.trie_compile_lists(h, *W.pack(toks), len(toks))
+    off, tok = T.trie_copy_lists(h)
+    host = torch.full((len(tok),), -5, dtype=torch.int32, pin_memory=True)
+    rc = h._lib.trie_copy_lists(h.handle, None, ctypes.c_void_p(host.data_ptr()),
+                                ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    torch.cuda.synchronize()
+    assert rc == 0 and torch.equal(host, tok.cpu())
