@@ -842,7 +842,8 @@ int trie_advance_apply(trie_t h, const int32_t *d_states_in, const int32_t *d_to
     if ((rc = current_device(&dev)) != TRIE_OK) return rc;
     if (dev != h->dev.device) return fail(TRIE_EINVAL, "handle belongs to another device");
     cudaError_t e = tmk::launch_advance_apply(h->dev, h->host.n, *voc, use_trans, d_states_in, d_tokens,
-                                              d_states_out, d_err, d_logits, dtype, mask, B, stream, seg);
+                                              d_states_out, d_err, d_logits, dtype, mask, B, num_sms(dev),
+                                              stream, seg);
     if (e != cudaSuccess) return fail_cuda(e, "advance-apply launch");
     return TRIE_OK;
 }
@@ -870,7 +871,7 @@ int trie_apply_mask(trie_t h, void *d_logits, int dtype, const int32_t *d_states
     int dev, rc;
     if ((rc = current_device(&dev)) != TRIE_OK) return rc;
     if (dev != h->dev.device) return fail(TRIE_EINVAL, "handle belongs to another device");
-    cudaError_t e = tmk::launch_apply(d_logits, dtype, mask, d_states, B, V, h->host.n, stream, seg);
+    cudaError_t e = tmk::launch_apply(d_logits, dtype, mask, d_states, B, V, h->host.n, num_sms(dev), stream, seg);
     if (e != cudaSuccess) return fail_cuda(e, "apply launch");
     return TRIE_OK;
 }
@@ -1485,7 +1486,7 @@ int fmt_apply_mask(fmt_t f, void *d_logits, int dtype, const int32_t *d_states, 
     int dev, rc;
     if ((rc = current_device(&dev)) != TRIE_OK) return rc;
     if (dev != f->device) return fail(TRIE_EINVAL, "handle belongs to another device");
-    cudaError_t e = tmk::launch_apply(d_logits, dtype, mask, d_states, B, V, f->L + 1, stream);
+    cudaError_t e = tmk::launch_apply(d_logits, dtype, mask, d_states, B, V, f->L + 1, num_sms(dev), stream);
     if (e != cudaSuccess) return fail_cuda(e, "format apply launch");
     return TRIE_OK;
 }

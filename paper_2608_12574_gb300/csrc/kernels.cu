@@ -906,7 +906,15 @@ __global__ void __launch_bounds__(kPairwiseThreads) k_mask_pairwise(AdvanceArgs 
 
 // ------------------------------------------------------------------ apply
 
+// CTAs of the applies: 256 threads, or 128 for launches of at most
+// kApplySmallItems segments an SM, whose time is mostly that of one CTA from
+// launch to end (a loop's step at V = 32,000, fp32: B = 1 1.93 and 1.76 us, B =
+// 16 2.53 and 2.32 us; at V = 262,144, B = 8 3.84 and 3.60 us). Above that 128
+// threads gain nothing or lose (V = 262,144, fp32, B = 16 4.13 against 4.25 us;
+// V = 152,064, bf16, B = 256 11.9 against 12.1 us).
 constexpr int kApplyThreads = 256;
+constexpr int kApplySmallThreads = 128;
+constexpr int64_t kApplySmallItems = 24;  // segments per SM
 
 // Mask word of (state, word index w): the node's row, or {EOS} for FINISHED,
 // DEAD and ids that are not nodes.
@@ -1083,10 +1091,10 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_vec(void *__restrict__ 
                                                              int32_t segs, SegRef sg) {
     constexpr int kSegChunks = 1024 / (16 / kElt);
     __shared__ __align__(128) uint4 tile[kSegChunks];
-    init_ninf_tile<kElt>(tile);
     pdl_launch_dependents();
+    init_ninf_tile<kElt>(tile);
     const int lane = threadIdx.x & 31;
-    const int64_t item = int64_t(blockIdx.x) * (kApplyThreads / 32) + (threadIdx.x >> 5);
+    const int64_t item = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int32_t b = item <= INT32_MAX ? int32_t(item) / segs : int32_t(item / segs);
     const int32_t seg = int32_t(item - int64_t(b) * segs);
     const RowCut<kElt> row(logits, b, V);
@@ -1098,7 +1106,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_vec(void *__restrict__ 
 // Advance, then apply, in one launch (one decode step once the sampler has
 // picked tokens[b] for the previous logits): states_out[b] = delta*(states_in[b],
 // tokens[b]), and logits[b] (the next step's) are masked by the row of
-// states_out[b]. CTA (row b, part p) covers segments 8p .. 8p + 7 of row b,
+// states_out[b]. CTA (row b, part p) covers the p-th run of segments of row b,
 // one warp each; its thread 0 computes the row's new state once for the CTA
 // (shared memory), and the CTA of part 0 stores it and counts a move into
 // DEAD.
@@ -1134,7 +1142,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_advance_apply_vec(AdvanceArgs
     __syncthreads();
     pdl_wait();  // logits come from earlier kernels
     const int lane = threadIdx.x & 31;
-    const int32_t seg = part * (kApplyThreads / 32) + int32_t(threadIdx.x >> 5);
+    const int32_t seg = part * int32_t(blockDim.x >> 5) + int32_t(threadIdx.x >> 5);
     if (seg >= segs) return;  // uniform per warp
     mask_segment<kElt>(row, aa.V, mask, sg, epoch, next_state, aa.n_nodes, W, seg, lane, tile);
 }
@@ -1432,13 +1440,13 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_lists(void *__restrict_
     __shared__ __align__(128) uint4 tile[kSegChunks];
     __shared__ uint32_t words[kWords], head_bits;
     __shared__ int32_t state, moved;
+    pdl_launch_dependents();
     for (int i = threadIdx.x; i < kWords; i += kApplyThreads) words[i] = 0u;
     if (threadIdx.x == 0) {
         moved = kDead;
         head_bits = 0u;
     }
     init_ninf_tile<kElt>(tile);
-    pdl_launch_dependents();
     const int32_t b = int32_t(blockIdx.x) / parts, part = int32_t(blockIdx.x) - b * parts;
     const RowCut<kElt> row(logits, b, V);
     pdl_wait();  // logits, states and tokens come from earlier kernels
@@ -2095,40 +2103,51 @@ cudaError_t launch_advance(const DevTrie &t, int32_t n_nodes, const DevVocab &v,
                       states_out, tokens, B, err);
 }
 
+namespace {
+
+// Threads per CTA of an apply over B rows of `segs` segments.
+int apply_threads(int64_t B, int32_t segs, int num_sms) {
+    return B * segs <= kApplySmallItems * int64_t(num_sms) ? kApplySmallThreads : kApplyThreads;
+}
+
+}  // namespace
+
 cudaError_t launch_advance_apply(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bool use_trans,
                                  const int32_t *states_in, const int32_t *tokens, int32_t *states_out,
                                  int32_t *err, void *logits, int dtype, const uint32_t *mask, int32_t B,
-                                 cudaStream_t st, const SegRef &seg) {
+                                 int num_sms, cudaStream_t st, const SegRef &seg) {
     const int32_t V = v.V;
     const int64_t W = (int64_t(V) + 31) / 32;
     const int elt = dtype == 0 ? 4 : 2;
     const int32_t segs = int32_t((W + 31) / 32);
-    const int32_t parts = (segs + kApplyThreads / 32 - 1) / (kApplyThreads / 32);
+    const int threads = apply_threads(B, segs, num_sms);
+    const int32_t parts = (segs + threads / 32 - 1) / (threads / 32);
     const int64_t grid = int64_t(B) * parts;
     if (grid > INT32_MAX) {  // more CTAs than a grid holds: the two kernels one after the other
         cudaError_t e = launch_advance(t, n_nodes, v, states_in, states_out, tokens, B, err, use_trans, st);
         if (e != cudaSuccess) return e;
-        return launch_apply(logits, dtype, mask, states_out, B, V, n_nodes, st, seg);
+        return launch_apply(logits, dtype, mask, states_out, B, V, n_nodes, num_sms, st, seg);
     }
     const AdvanceArgs aa = advance_args(t, n_nodes, v, use_trans);
     if (elt == 2)
-        return launch_pdl(k_advance_apply_vec<2>, grid, kApplyThreads, st, aa, logits, mask, states_in, tokens,
+        return launch_pdl(k_advance_apply_vec<2>, grid, threads, st, aa, logits, mask, states_in, tokens,
                           states_out, err, B, W, segs, parts, seg);
-    return launch_pdl(k_advance_apply_vec<4>, grid, kApplyThreads, st, aa, logits, mask, states_in, tokens,
+    return launch_pdl(k_advance_apply_vec<4>, grid, threads, st, aa, logits, mask, states_in, tokens,
                       states_out, err, B, W, segs, parts, seg);
 }
 
 cudaError_t launch_apply(void *logits, int dtype, const uint32_t *mask, const int32_t *states,
-                         int32_t B, int32_t V, int32_t n_nodes, cudaStream_t st, const SegRef &seg) {
+                         int32_t B, int32_t V, int32_t n_nodes, int num_sms, cudaStream_t st, const SegRef &seg) {
     const int64_t W = (int64_t(V) + 31) / 32;
     const int32_t segs = int32_t((W + 31) / 32);
     // more CTAs than a grid holds would mean more logits than any device does
-    const int64_t grid = (int64_t(B) * segs + kApplyThreads / 32 - 1) / (kApplyThreads / 32);
+    const int threads = apply_threads(B, segs, num_sms);
+    const int64_t grid = (int64_t(B) * segs + threads / 32 - 1) / (threads / 32);
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
     if (dtype == 0)
-        return launch_pdl(k_apply_vec<4>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes, segs,
+        return launch_pdl(k_apply_vec<4>, grid, threads, st, logits, mask, states, B, V, W, n_nodes, segs,
                           seg);
-    return launch_pdl(k_apply_vec<2>, grid, kApplyThreads, st, logits, mask, states, B, V, W, n_nodes, segs, seg);
+    return launch_pdl(k_apply_vec<2>, grid, threads, st, logits, mask, states, B, V, W, n_nodes, segs, seg);
 }
 
 namespace {
@@ -2338,7 +2357,7 @@ cudaError_t launch_lazy(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bo
     e = launch_pdl_smem(k_lazy_rows, rows_grid, kLazyRowThreads, size_t(L.W) * sizeof(uint32_t), st, la, pa);
     if (e != cudaSuccess) return e;
     const int32_t n_rows = L.C + L.max_batch;
-    if (logits) return launch_apply(logits, dtype, L.rows, L.slot_of, B, L.V, n_rows, st);
+    if (logits) return launch_apply(logits, dtype, L.rows, L.slot_of, B, L.V, n_rows, num_sms, st);
     const int grid = grid_for(int64_t(B) * L.W, kApplyThreads, int64_t(num_sms) * 8);
     return launch_pdl(k_lazy_gather, grid, kApplyThreads, st, static_cast<const uint32_t *>(L.rows),
                       static_cast<const int32_t *>(L.slot_of), B, L.W, n_rows, L.V - 1, rows_out);

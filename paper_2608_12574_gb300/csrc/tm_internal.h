@@ -476,9 +476,9 @@ cudaError_t launch_advance(const DevTrie &t, int32_t n_nodes, const DevVocab &v,
 cudaError_t launch_advance_apply(const DevTrie &t, int32_t n_nodes, const DevVocab &v, bool use_trans,
                                  const int32_t *states_in, const int32_t *tokens, int32_t *states_out,
                                  int32_t *err, void *logits, int dtype, const uint32_t *mask, int32_t B,
-                                 cudaStream_t st, const SegRef &seg);
+                                 int num_sms, cudaStream_t st, const SegRef &seg);
 cudaError_t launch_apply(void *logits, int dtype, const uint32_t *mask, const int32_t *states,
-                         int32_t B, int32_t V, int32_t n_nodes, cudaStream_t st,
+                         int32_t B, int32_t V, int32_t n_nodes, int num_sms, cudaStream_t st,
                          const SegRef &seg = SegRef());
 // Copies (d_k, s_k, b_k bytes), k = 0..2, in one launch; the sources are read
 // by the kernel itself (device memory, or host memory the device reads

@@ -73,10 +73,11 @@ def test_apply_row_cuts(cuda, V, dtype):
                 assert np.array_equal(ds1.cpu().numpy(), s1)
 
 
-@pytest.mark.parametrize("V", [32767, 65533])
-def test_apply_summary_unaligned(cuda, V):
+@pytest.mark.parametrize("V,B", [(32767, 32), (65533, 32), (65533, 120)])
+def test_apply_summary_unaligned(cuda, V, B):
     """Unaligned rows of a mask with a segment summary whose words are full (32
-    or 64 segments): the last segment has no next one to take bits from."""
+    or 64 segments): the last segment has no next one to take bits from. 120
+    rows take CTAs of 256 threads, 32 rows CTAs of 128."""
     import torch
     names = W.tool_names(1, 1000, 200)
     sb, so = W.pack(names)
@@ -88,7 +89,7 @@ def test_apply_summary_unaligned(cuda, V):
     ot, ov = oracle.Trie(sb, so), oracle.Vocab(vb, vo)
     rng = np.random.default_rng(V)
     n = h.num_nodes
-    s0 = np.concatenate([[0, n - 1, n - 2, -1, -2], rng.integers(0, n, 32)]).astype(np.int32)
+    s0 = np.concatenate([[0, n - 1, n - 2, -1, -2], rng.integers(0, n, B)]).astype(np.int32)
     raw = rng.integers(0, 2 ** 16, (len(s0), V), dtype=np.uint32).astype(np.uint16)
     want = oracle.apply(ot, ov, raw, s0)
     x = torch.from_numpy(raw.view(np.int16)).view(torch.bfloat16).to(cuda)
