@@ -187,6 +187,30 @@ int get_vocab(const uint8_t *vb, const int64_t *vo, int32_t V, int dev,
 // Uploads the trie on first use, ordered on `stream` (the copies read the
 // handle's own host arrays, which outlive them); the handle is bound to that
 // device.
+// The segment summary of the dense mask (bit g of row r set iff the row allows
+// a token of the 1,024-token segment g), which lets the apply skip reading
+// the mask words of empty segments; none when it would exceed 256 MB, and
+// none for tries of more than kSegMaxNodes nodes: the probe sets the summary
+// while the fill runs, and for a forest of millions of nodes its
+// compare-and-swaps made it outlast the fill (dense compile of the 4.77 M-node
+// forest 12.9 ms with the summary, 11.1 ms without).
+constexpr int32_t kSegMaxNodes = int32_t(1) << 18;
+constexpr size_t kSegHead = 16;  // the epoch word, before the summary words
+bool seg_fits(int64_t n, int32_t words) { return n <= kSegMaxNodes && n * words * 8 <= (int64_t(256) << 20); }
+
+// (epoch 0 is never a compile's: with cleared memory every word starts out empty)
+void place_seg(tmk::DevTrie *t, char *p, int64_t words) {
+    t->seg_epoch = reinterpret_cast<uint32_t *>(p);
+    t->seg_any = reinterpret_cast<unsigned long long *>(p + kSegHead);
+    t->seg_cap = words;
+}
+
+// Device memory to be cleared when a trie is uploaded.
+struct ClearRange {
+    void *p = nullptr;
+    size_t bytes = 0;
+};
+
 // Places the per-node compile tables (window, depth16, anc) in a layout.
 struct TableLayout {
     size_t win, d16, anc;
@@ -203,8 +227,12 @@ struct TableLayout {
 // single: a single trie, which gets the compile tables at once and a
 // transition table (8 or more slots per node) for the compiles to record
 // moves in. A forest gets the tables on its first dense compile or lazy
-// set-up (ensure_tables): its valid lists need neither.
-int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool single) {
+// set-up (ensure_tables): its valid lists need neither. dense_words: the words
+// per row of the segment summary where the upload is for a dense compile of a
+// single trie, which then also gets the hit buffer and the summary here (one
+// allocation instead of three); else 0.
+int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool single, int32_t dense_words,
+                      ClearRange *clear) {
     Layout L;
     const size_t o_par = L.add(sizeof(int32_t) * n);
     const size_t o_lab = L.add(n);
@@ -214,11 +242,24 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool sin
     const TableLayout tables(L, single ? n : 0);
     size_t trans_slots = single ? 16 : 0;  // >= 8 per node, a power of two
     while (single && trans_slots < 8 * n) trans_slots <<= 1;
+    const bool dense = single && dense_words > 0;
+    const int64_t seg_words = dense && seg_fits(int64_t(n), dense_words) ? int64_t(n) * dense_words : 0;
+    const size_t o_hits = L.add(dense ? sizeof(int2) * tmk::kHitSlots * n : 0);
+    const size_t o_hcnt = L.add(dense ? n : 0);
     const size_t o_trans = L.add(sizeof(ulonglong2) * trans_slots);
+    const size_t o_seg = L.add(seg_words ? kSegHead + size_t(seg_words) * 8 : 0);
     void *base = nullptr;
     const int rc = pool_alloc(dev, L.total, stream, &base, "the trie");
     if (rc != TRIE_OK) return rc;
     char *b = static_cast<char *>(base);
+    if (dense) {  // the transition table and the summary behind it start out cleared
+        h->dev.hits = reinterpret_cast<int2 *>(b + o_hits);
+        h->dev.hit_count = reinterpret_cast<uint8_t *>(b + o_hcnt);
+        if (seg_words) place_seg(&h->dev, b + o_seg, seg_words);
+        h->dev.trans_clean = true;
+        clear->p = b + o_trans;
+        clear->bytes = L.total - o_trans;
+    }
     h->dev.device = dev;
     h->dev.base = base;
     h->dev.parent = reinterpret_cast<const int32_t *>(b + o_par);
@@ -234,9 +275,10 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool sin
 
 // The child links, and a single trie's compile tables, from the device's
 // parent / label / terminal arrays (once they are written on `stream`).
-int finish_device_trie(trie_t h, int dev, cudaStream_t stream) {
-    cudaError_t e = tmk::launch_trie_links(h->dev, h->host.n, num_sms(dev), stream);
-    if (e == cudaSuccess && h->dev.window) e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
+int finish_device_trie(trie_t h, int dev, cudaStream_t stream, const ClearRange &clear) {
+    const cudaError_t e =
+        h->dev.window ? tmk::launch_trie_setup(h->dev, h->host.n, clear.p, clear.bytes, num_sms(dev), stream)
+                      : tmk::launch_trie_links(h->dev, h->host.n, num_sms(dev), stream);
     if (e != cudaSuccess) {
         pool_free(h->dev.base);
         h->dev = tmk::DevTrie();
@@ -270,7 +312,8 @@ int ensure_tables(trie_t h, int dev, cudaStream_t stream) {
 
 bool host_memory_direct(int dev);
 
-int ensure_device_trie(trie_t h, int dev, cudaStream_t stream) {
+// dense_words: as in alloc_device_trie.
+int ensure_device_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_words = 0) {
     std::lock_guard<std::mutex> lk(h->mu);
     if (h->dev.base) {
         if (h->dev.device != dev)
@@ -282,7 +325,8 @@ int ensure_device_trie(trie_t h, int dev, cudaStream_t stream) {
     const size_t n = size_t(t.n);
     // a transition table for a single trie; a forest's per-request sets are
     // decoded for a few steps, where byte walks cost less than the table
-    int rc = alloc_device_trie(h, dev, n, stream, t.roots.size() <= 1);
+    ClearRange clear;
+    int rc = alloc_device_trie(h, dev, n, stream, t.roots.size() <= 1, dense_words, &clear);
     if (rc != TRIE_OK) return rc;
     if (host_memory_direct(dev)) {
         // the kernel reads the handle's host arrays itself: a pageable copy
@@ -296,7 +340,7 @@ int ensure_device_trie(trie_t h, int dev, cudaStream_t stream) {
             h->dev = tmk::DevTrie();
             return fail_cuda(e, "uploading the trie");
         }
-        return finish_device_trie(h, dev, stream);
+        return finish_device_trie(h, dev, stream, clear);
     }
     struct Up { const void *dst; const void *src; size_t n; } ups[] = {
         {h->dev.parent, t.parent.data(), sizeof(int32_t) * n},
@@ -311,7 +355,7 @@ int ensure_device_trie(trie_t h, int dev, cudaStream_t stream) {
             return fail_cuda(e, "uploading the trie");
         }
     }
-    return finish_device_trie(h, dev, stream);
+    return finish_device_trie(h, dev, stream, clear);
 }
 
 // The transition table holds transitions of one vocabulary: when a compile
@@ -327,8 +371,11 @@ int prepare_trans(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, int sms, 
     }
     h->trans_vocab.reset();
     h->trans_complete = false;
-    cudaError_t e = tmk::launch_trans_clear(h->dev, sms, stream);
-    if (e != cudaSuccess) return fail_cuda(e, "transition table clear");
+    if (!h->dev.trans_clean) {
+        cudaError_t e = tmk::launch_trans_clear(h->dev, sms, stream);
+        if (e != cudaSuccess) return fail_cuda(e, "transition table clear");
+    }
+    h->dev.trans_clean = false;
     *fill = true;
     return TRIE_OK;
 }
@@ -591,7 +638,8 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
             h->host_arrays = false;
             // per-batch sets are decoded for a few steps: no transition
             // table to clear and fill (advance walks the tokens' bytes)
-            if ((rc = alloc_device_trie(h, dev, size_t(n), stream, false)) != TRIE_OK) {
+            ClearRange none;
+            if ((rc = alloc_device_trie(h, dev, size_t(n), stream, false, 0, &none)) != TRIE_OK) {
                 delete h;
                 return rc;
             }
@@ -601,7 +649,7 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
     } catch (const std::bad_alloc &) {
         e = cudaErrorMemoryAllocation;
     }  // the scratch is freed on the stream after the last kernel
-    if (e == cudaSuccess && (rc = finish_device_trie(h, dev, stream)) != TRIE_OK) {
+    if (e == cudaSuccess && (rc = finish_device_trie(h, dev, stream, ClearRange())) != TRIE_OK) {
         delete h;
         return rc;
     }
@@ -662,7 +710,7 @@ int trie_get_csr(trie_t h, int32_t *parent, uint8_t *label, uint8_t *terminal, i
 // never need it, so a forest compiled to lists does not hold 129 B per node.
 static int ensure_hits(trie_t h, int dev, cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(h->mu);
-    if (h->dev.hits_base) return TRIE_OK;
+    if (h->dev.hits) return TRIE_OK;
     const size_t n = size_t(h->host.n);
     Layout L;
     const size_t o_hits = L.add(sizeof(int2) * tmk::kHitSlots * n);
@@ -677,38 +725,31 @@ static int ensure_hits(trie_t h, int dev, cudaStream_t stream) {
     return TRIE_OK;
 }
 
-// The segment summary of the dense mask (bit g of row r set iff the row allows
-// a token of the 1,024-token segment g), which lets the apply skip reading
-// the mask words of empty segments; none when it would exceed 256 MB, and
-// none for tries of more than kSegMaxNodes nodes: the probe sets the summary
-// while the fill runs, and for a forest of millions of nodes its
-// compare-and-swaps made it outlast the fill (dense compile of the 4.77 M-node
-// forest 12.9 ms with the summary, 11.1 ms without).
-constexpr int32_t kSegMaxNodes = int32_t(1) << 18;
+// The handle's segment summary, allocated here where the upload has not (or
+// for fewer words).
 static unsigned long long *ensure_seg(trie_t h, int dev, cudaStream_t stream, int32_t words) {
     const int64_t need = int64_t(h->host.n) * words;
-    if (need * 8 > (int64_t(256) << 20)) return nullptr;
+    if (!seg_fits(h->host.n, words)) return nullptr;
     std::lock_guard<std::mutex> lk(h->mu);
     if (h->dev.seg_cap < need) {
-        pool_free(h->dev.seg_epoch);  // an earlier apply may still read it
+        pool_free(h->dev.seg_base);  // an earlier apply may still read it
+        h->dev.seg_base = nullptr;
         h->dev.seg_any = nullptr;
         h->dev.seg_epoch = nullptr;
         h->dev.seg_cap = 0;
         void *p = nullptr;
-        const size_t bytes = 16 + size_t(need) * 8;  // the epoch word, then the summary words
+        const size_t bytes = kSegHead + size_t(need) * 8;
         if (pool_alloc(dev, bytes, stream, &p, "the mask's segment summary") != TRIE_OK) {
             cudaGetLastError();
             return nullptr;  // the compile and the apply work without it
         }
-        // epoch 0 is never a compile's: every word starts out empty
         if (cudaMemsetAsync(p, 0, bytes, stream) != cudaSuccess) {
             cudaGetLastError();
             pool_free(p);
             return nullptr;
         }
-        h->dev.seg_epoch = static_cast<uint32_t *>(p);
-        h->dev.seg_any = reinterpret_cast<unsigned long long *>(static_cast<char *>(p) + 16);
-        h->dev.seg_cap = need;
+        h->dev.seg_base = p;
+        place_seg(&h->dev, static_cast<char *>(p), need);
     }
     return h->dev.seg_any;
 }
@@ -718,17 +759,17 @@ static int compile_masks(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
                          cudaStream_t stream) {
     int rc;
     const int32_t V = voc->V;
-    if ((rc = ensure_device_trie(h, dev, stream)) != TRIE_OK) return rc;
+    const int64_t W = (int64_t(V) + 31) / 32;
+    const int32_t seg_words = int32_t(((W + 31) / 32 + 31) / 32);
+    if ((rc = ensure_device_trie(h, dev, stream, seg_words)) != TRIE_OK) return rc;
     if ((rc = ensure_tables(h, dev, stream)) != TRIE_OK) return rc;
     if ((rc = ensure_hits(h, dev, stream)) != TRIE_OK) return rc;
-    const int64_t W = (int64_t(V) + 31) / 32;
     const int32_t n = h->host.n;
     const int32_t lmax = std::min(voc->max_len, h->host.max_depth);
     const int sms = num_sms(dev);
     bool fill_trans;
     if ((rc = prepare_trans(h, voc, sms, stream, &fill_trans)) != TRIE_OK) return rc;
-    const int32_t seg_words = int32_t(((W + 31) / 32 + 31) / 32);
-    unsigned long long *seg = n <= kSegMaxNodes ? ensure_seg(h, dev, stream, seg_words) : nullptr;
+    unsigned long long *seg = ensure_seg(h, dev, stream, seg_words);
     const uint32_t epoch = h->dev.seg_epoch_next;
     h->dev.seg_epoch_next = epoch == UINT32_MAX ? 1u : epoch + 1u;
     bool seg_written = false;
@@ -1255,8 +1296,9 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
         if (h->dev.trans && h->trans_vocab != voc) {
             h->trans_vocab.reset();
             h->trans_complete = false;
-            if ((e = tmk::launch_trans_clear(h->dev, num_sms(dev), 0)) != cudaSuccess)
+            if (!h->dev.trans_clean && (e = tmk::launch_trans_clear(h->dev, num_sms(dev), 0)) != cudaSuccess)
                 return fail_cuda(e, "transition table clear");
+            h->dev.trans_clean = false;
             h->trans_vocab = voc;
         }
     }
@@ -1517,7 +1559,7 @@ int trie_destroy(trie_t h) {
         }
         pool_free(h->dev.hits_base);
         pool_free(h->dev.tables_base);
-        pool_free(h->dev.seg_epoch);
+        pool_free(h->dev.seg_base);
         pool_free(h->dev.base);
         if (h->lists.done) cudaEventDestroy(h->lists.done);
     }
@@ -1596,7 +1638,7 @@ int trie_destroy_async(trie_t h, cudaStream_t stream) {
         }
         free_on(h->dev.hits_base);
         free_on(h->dev.tables_base);
-        free_on(h->dev.seg_epoch);
+        free_on(h->dev.seg_base);
         free_on(h->dev.base);
         // the event may still be pending: CUDA defers its destruction
         if (h->lists.done) cudaEventDestroy(h->lists.done);

@@ -255,17 +255,19 @@ struct DevTrie {
     int4 *anc = nullptr;             // [n * 4]
     ulonglong2 *trans = nullptr;     // transition table {(row << 32 | token) + 1, end node}
     uint32_t trans_mask = 0;         // slots - 1
+    bool trans_clean = false;        // the table was cleared at the upload and not used since
     // Segment summary of the dense mask (own allocation): per row, words of 32
     // segment bits (1,024 tokens each) tagged in their high half with the
     // epoch of the compile that set them; a word with another tag than the
     // device's current epoch (*seg_epoch, written by each compile's probe)
     // holds no allowed token.
     unsigned long long *seg_any = nullptr;  // seg_cap words
+    void *seg_base = nullptr;               // epoch and words, when allocated after the upload
     uint32_t *seg_epoch = nullptr;          // [1] (device), the epoch of the last compile that ran
     uint32_t seg_epoch_next = 1;            // host: the epoch of the next compile (0 is never used)
     int64_t seg_cap = 0;
     void *tables_base = nullptr;     // a forest's window, depth16 and anc (own allocation)
-    void *hits_base = nullptr;       // the two arrays below (allocated by the first dense compile)
+    void *hits_base = nullptr;       // the two arrays below, when allocated after the upload
     int2 *hits = nullptr;            // compile scratch: kHitSlots (row, token) pairs per node
     uint8_t *hit_count = nullptr;    // compile scratch: hits found per node
 };
@@ -463,6 +465,10 @@ cudaError_t launch_mask_compile3(const DevTrie &t, int32_t n_nodes, const DevVoc
 // Writes every entry of t.first_child (-1 for a leaf) and t.child_bits from
 // t.parent and t.label; nothing needs clearing first (tables.cu).
 cudaError_t launch_trie_links(const DevTrie &t, int32_t n_nodes, int num_sms, cudaStream_t st);
+// Both of a single trie in one launch (tables.cu), and clear_bytes (a multiple
+// of 16) of cleared memory at clear.
+cudaError_t launch_trie_setup(const DevTrie &t, int32_t n_nodes, void *clear, size_t clear_bytes, int num_sms,
+                              cudaStream_t st);
 // Fills t.window, t.depth16 and t.anc from t.parent and t.label (tables.cu).
 cudaError_t launch_trie_tables(const DevTrie &t, int32_t n_nodes, int num_sms, cudaStream_t st);
 // Zeroes the transition table (before it is filled for another vocabulary).
