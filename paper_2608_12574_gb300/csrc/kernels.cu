@@ -1546,7 +1546,8 @@ __device__ __forceinline__ int32_t lazy_set(int32_t s, int32_t n_sets) {
 // thread keeps its batch rows' results in registers and the missing nodes stay
 // in shared memory, so nothing is passed on through L2 between the phases
 // (K = 10,000, B = 256, no cache: 6.7-7.1 us of a step from the apply before
-// to its end, 4.6-6.4 us so).
+// to its end, 4.6-6.4 us so; without a cache, tasks added by whoever enters a
+// node in the first phase gained nothing).
 constexpr int kResolvePer = kLazyMaxBatch / kResolveThreads;  // batch rows per thread
 
 template <bool kAdvance>
@@ -1662,16 +1663,23 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
         }
         const int32_t t0 = atomicAdd(&n_tasks, parts);
         const int32_t k = place.x + 1;
+        LazyTask t;
+        t.node = s;
+        t.row = row;
+        t.pos = place.x;
+        t.part = 0;
+        t.k0 = k;
+        t.k1 = k + desc;
+        t.parts = parts;
+        t.pad = 0;
+        if (parts == 1) {
+            L.task[t0] = t;
+            continue;
+        }
         for (int32_t p = 0; p < parts; p++) {
-            LazyTask t;
-            t.node = s;
-            t.row = row;
-            t.pos = place.x;
             t.part = p;
             t.k0 = k + int32_t(int64_t(desc) * p / parts);
             t.k1 = k + int32_t(int64_t(desc) * (p + 1) / parts);
-            t.parts = parts;
-            t.pad = 0;
             L.task[t0 + p] = t;
         }
     }
@@ -1680,7 +1688,12 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
     const int32_t n_zero = n_split < kLazySplitRows ? n_split : kLazySplitRows;
     for (int32_t r = 0; r < n_zero; r++) {
         uint32_t *row = L.rows + int64_t(split_slot[r]) * L.W;
-        for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) row[i] = 0u;
+        if ((L.W & 3) == 0) {  // rows start on 16-byte boundaries
+            for (int64_t i = threadIdx.x; i < L.W / 4; i += blockDim.x)
+                reinterpret_cast<uint4 *>(row)[i] = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+            for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) row[i] = 0u;
+        }
     }
     // 3. every batch row's cache row
 #pragma unroll
@@ -1692,8 +1705,8 @@ __global__ void __launch_bounds__(kResolveThreads) k_lazy_resolve(LazyArgs L, Ad
         L.ctrl->n_miss = n_u;
         L.ctrl->n_tasks = n_tasks;
         L.ctrl->now = now + 1u;
-        L.ctrl->hits += n_hit;
-        L.ctrl->misses += n_miss_rows;
+        atomicAdd(&L.ctrl->hits, static_cast<unsigned long long>(n_hit));  // nothing to wait for
+        atomicAdd(&L.ctrl->misses, static_cast<unsigned long long>(n_miss_rows));
     }
 }
 
@@ -1722,8 +1735,12 @@ __device__ __forceinline__ uint64_t hash_pow(uint32_t j) {
 // again and the token's id, length and bytes one after the other, 7.8-9.4 us
 // so). The moves it found are kept until the row is stored: inserted as they
 // are found, each one's compare-and-swap in the transition table held up the
-// row. (Moves beyond the list are inserted at once.)
+// row. (Moves beyond the list are inserted at once. A look at the slot before
+// the compare-and-swap gained nothing.) The first task is read beside the
+// tasks' count, whole rows are stored 16 bytes at a time, and the powers of the
+// hash's base come from shared memory: 24.2 us a step before these, 23.4 us so.
 constexpr int kLazyMoves = 256;
+constexpr int kLazyPows = 32;  // powers of the hash's base kept in shared memory
 
 // The tokens on the paths from s (at depth d0, path hash ps) down to the
 // descendants at pre-order positions k0 .. k1 - 1: their bits, and the moves
@@ -1734,8 +1751,8 @@ constexpr int kLazyMoves = 256;
 // us).
 template <int G>
 __device__ __forceinline__ void search_descendants(const LazyArgs &L, const PatchArgs &a, int32_t s, uint64_t ps,
-                                                   int32_t d0, int32_t k0, int32_t k1, uint32_t *bits, int2 *moves,
-                                                   int32_t *n_moves) {
+                                                   int32_t d0, int32_t k0, int32_t k1, const uint64_t *pow,
+                                                   uint32_t *bits, int2 *moves, int32_t *n_moves) {
     const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(a.ht_key);
     const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
     for (int32_t kb = k0 + int32_t(threadIdx.x); kb < k1; kb += G * blockDim.x) {
@@ -1763,7 +1780,8 @@ __device__ __forceinline__ void search_descendants(const LazyArgs &L, const Patc
         ulonglong2 f[G];
 #pragma unroll
         for (int g = 0; g < G; g++) {
-            key[g] = hash_finish(pd[g] - ps * hash_pow(uint32_t(j[g])), uint32_t(j[g]));
+            const uint64_t bj = j[g] < kLazyPows ? pow[j[g]] : hash_pow(uint32_t(j[g]));
+            key[g] = hash_finish(pd[g] - ps * bj, uint32_t(j[g]));
             f[g] = j[g] > 0 ? __ldg(pairs + (uint32_t(key[g] >> 1) & a.pairs_mask)) : make_ulonglong2(0ull, 0ull);
         }
         // keys are resolved together (find_slots); paths longer than the
@@ -1843,34 +1861,48 @@ __device__ __forceinline__ void search_descendants(const LazyArgs &L, const Patc
 }
 
 __global__ void __launch_bounds__(kLazyRowThreads, 2) k_lazy_rows(LazyArgs L, PatchArgs a) {
-    extern __shared__ uint32_t bits[];
+    extern __shared__ __align__(16) uint32_t bits[];
     __shared__ int2 moves[kLazyMoves];  // {token, end node}
     __shared__ int32_t n_moves;
+    __shared__ uint64_t pow[kLazyPows];
     pdl_launch_dependents();
+    if (threadIdx.x < kLazyPows) pow[threadIdx.x] = hash_pow(threadIdx.x);
     for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) bits[i] = 0u;
     if (threadIdx.x == 0) n_moves = 0;
     pdl_wait();  // the resolve's task list
     const int32_t n_tasks = __ldcg(&L.ctrl->n_tasks);
     const ulonglong2 *rec = reinterpret_cast<const ulonglong2 *>(L.pre);  // 2 per record
+    const int4 *task = reinterpret_cast<const int4 *>(L.task);            // 2 per task
+    int4 t0 = __ldcg(task + 2 * blockIdx.x), t1 = __ldcg(task + 2 * blockIdx.x + 1);  // beside the count
     for (int32_t ti = blockIdx.x; ti < n_tasks; ti += gridDim.x) {
-        const int4 t0 = __ldcg(reinterpret_cast<const int4 *>(L.task + ti));
-        const int4 t1 = __ldcg(reinterpret_cast<const int4 *>(L.task + ti) + 1);
+        if (ti != int32_t(blockIdx.x)) {
+            t0 = __ldcg(task + 2 * ti);
+            t1 = __ldcg(task + 2 * ti + 1);
+        }
         const int32_t s = t0.x, slot_row = t0.y, pos = t0.z, part = t0.w, k0 = t1.x, k1 = t1.y, parts = t1.z;
         const ulonglong2 sh0 = __ldg(rec + 2 * int64_t(pos));
         const uint64_t ps = sh0.x;
         const int32_t d0 = int32_t(uint32_t(sh0.y));
         __syncthreads();  // bits and n_moves are zero
         if (threadIdx.x == 0 && part == 0 && __ldg(a.terminal + s)) atomicOr(bits + (a.eos >> 5), 1u << (a.eos & 31));
-        if (k1 - k0 <= kLazyRowThreads) search_descendants<1>(L, a, s, ps, d0, k0, k1, bits, moves, &n_moves);
-        else search_descendants<4>(L, a, s, ps, d0, k0, k1, bits, moves, &n_moves);
+        if (k1 - k0 <= kLazyRowThreads) search_descendants<1>(L, a, s, ps, d0, k0, k1, pow, bits, moves, &n_moves);
+        else search_descendants<4>(L, a, s, ps, d0, k0, k1, pow, bits, moves, &n_moves);
         __syncthreads();
         uint32_t *row = L.rows + int64_t(slot_row) * L.W;
         const int32_t kept = n_moves < kLazyMoves ? n_moves : kLazyMoves;
-        for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) {
-            const uint32_t w = bits[i];
-            if (parts == 1) row[i] = w;
-            else if (w) atomicOr(row + i, w);
-            bits[i] = 0u;  // for the CTA's next task
+        if (parts == 1 && (L.W & 3) == 0) {  // rows start on 16-byte boundaries
+            uint4 *b4 = reinterpret_cast<uint4 *>(bits);
+            for (int64_t i = threadIdx.x; i < L.W / 4; i += blockDim.x) {
+                reinterpret_cast<uint4 *>(row)[i] = b4[i];
+                b4[i] = make_uint4(0u, 0u, 0u, 0u);  // for the CTA's next task
+            }
+        } else {
+            for (int64_t i = threadIdx.x; i < L.W; i += blockDim.x) {
+                const uint32_t w = bits[i];
+                if (parts == 1) row[i] = w;
+                else if (w) atomicOr(row + i, w);
+                bits[i] = 0u;
+            }
         }
         for (int32_t i = threadIdx.x; i < kept; i += blockDim.x)
             trans_insert(a.trans, a.trans_mask, s, moves[i].x, moves[i].y);
