@@ -1288,9 +1288,11 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     if ((rc = get_vocab(vocab_bytes, vocab_offsets, V, dev, &voc)) != TRIE_OK) return rc;
     if ((rc = tmk::ensure_host_arrays(h)) != TRIE_OK) return rc;  // the pre-order tables
     if ((rc = ensure_device_trie(h, dev, 0)) != TRIE_OK) return rc;
-    if ((rc = ensure_tables(h, dev, 0)) != TRIE_OK) return rc;
-    cudaError_t e = cudaDeviceSynchronize();  // earlier lazy calls may still use the old cache
+    // earlier lazy calls may still use the old cache, and another stream may
+    // still be uploading or building the arrays that the tables come from
+    cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return fail_cuda(e, "synchronising before the lazy set-up");
+    if ((rc = ensure_tables(h, dev, 0)) != TRIE_OK) return rc;
     {  // the transition table takes the moves the lazy rows find for this vocabulary
         std::lock_guard<std::mutex> lk(h->mu);
         if (h->dev.trans && h->trans_vocab != voc) {

@@ -42,3 +42,28 @@ def test_tables_on_first_use(then, device_build, lists_first):
         m = T.trie_lazy_rows(h, torch.arange(h.num_nodes, dtype=torch.int32, device="cuda"), V)
     assert np.array_equal(m.cpu().numpy().view(np.uint32), want)
     (h.destroy_async if lists_first else h.destroy)()
+
+
+def test_lazy_setup_behind_an_upload_on_another_stream():
+    """The lists' upload waits on a busy stream while the lazy set-up asks for
+    the tables, which come from the arrays that it uploads."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    oracle.build()
+    strings, toks = random_case(91)
+    sb, so = W.pack(strings + strings[:3])
+    vb, vo = W.pack(toks)
+    V = len(toks)
+    h = T.trie_build_many(sb, so, np.array([0, len(strings), len(strings) + 3], np.int32))
+    ov = oracle.Vocab(vb, vo)
+    want = np.concatenate([oracle.mask_all(oracle.Trie(*W.pack(s)), ov) for s in (strings, strings[:3])])
+    voc = T.trie_vocab_create(vb, vo, V)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)  # about 10 ms
+        T.trie_compile_lists_vocab(h, voc, side, count=False)
+    T.trie_lazy_init(h, vb, vo, V, cache_rows=0, max_batch=h.num_nodes)
+    m = T.trie_lazy_rows(h, torch.arange(h.num_nodes, dtype=torch.int32, device="cuda"), V)
+    assert np.array_equal(m.cpu().numpy().view(np.uint32), want)
+    h.destroy()
