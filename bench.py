@@ -580,7 +580,7 @@ def run_gpu(args, w, rank: int, world: int, dist):
                              "vs_suffix_search": pairwise_ms / compile_ms,
                              "kernel": "k_mask_pairwise (a lane per token walks it from the node; "
                                        "__ballot_sync per mask word)"},
-        "sparse_lists": {"entries": n_valid, "bytes": n_valid * 4 + (N + 1) * 8,
+        "sparse_lists": {"entries": n_valid, "bytes": n_valid * 8 + (N + 1) * 8,
                          "compile_ms": lists_ms,
                          "apply_us_avg": apply_lists_avg * 1e3,
                          "apply_gbs": (B * V * elt + B * 4) / (apply_lists_avg * 1e-3) / 1e9,
@@ -896,9 +896,9 @@ def run_dynamic(dev, stream, steps: int = 32, reps: int = 5, rank: int = 0, worl
     out["lists_compile_ms"] = min(lt)
     out["lists_compile_wall_ms"] = min(lw) * 1e3
     out["list_entries"] = n_valid
-    out["list_bytes"] = n_valid * 4 + (N + 1) * 8
-    # the list compile's algorithmic traffic: the entries and offsets written
-    # plus the trie's arrays the walks read (parent 4 B, label, terminal: 6 B
+    out["list_bytes"] = n_valid * 8 + (N + 1) * 8
+    # the list compile's algorithmic traffic: the entries (token and end node,
+    # 8 B) and offsets written plus the trie's arrays the walks read (parent 4 B, label, terminal: 6 B
     # per node, read by both walks)
     peak, peak_kind = peaks()
     list_bytes = out["list_bytes"] + 2 * 6 * N
