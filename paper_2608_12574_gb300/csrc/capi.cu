@@ -244,10 +244,13 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool sin
     while (single && trans_slots < 8 * n) trans_slots <<= 1;
     const bool dense = single && dense_words > 0;
     const int64_t seg_words = dense && seg_fits(int64_t(n), dense_words) ? int64_t(n) * dense_words : 0;
-    const size_t o_hits = L.add(dense ? sizeof(int2) * tmk::kHitSlots * n : 0);
-    const size_t o_hcnt = L.add(dense ? n : 0);
     const size_t o_trans = L.add(sizeof(ulonglong2) * trans_slots);
     const size_t o_seg = L.add(seg_words ? kSegHead + size_t(seg_words) * 8 : 0);
+    const size_t clear_end = L.total;
+    // the hit buffer last: between the tables and the transition table it cost
+    // the compile of K = 10,000 0.9 us (67.7 us, 66.8 us so and apart)
+    const size_t o_hits = L.add(dense ? sizeof(int2) * tmk::kHitSlots * n : 0);
+    const size_t o_hcnt = L.add(dense ? n : 0);
     void *base = nullptr;
     const int rc = pool_alloc(dev, L.total, stream, &base, "the trie");
     if (rc != TRIE_OK) return rc;
@@ -258,7 +261,7 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool sin
         if (seg_words) place_seg(&h->dev, b + o_seg, seg_words);
         h->dev.trans_clean = true;
         clear->p = b + o_trans;
-        clear->bytes = L.total - o_trans;
+        clear->bytes = clear_end - o_trans;
     }
     h->dev.device = dev;
     h->dev.base = base;
