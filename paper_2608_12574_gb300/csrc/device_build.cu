@@ -746,13 +746,16 @@ size_t nodes_smem(int32_t cap, int32_t D) {
 }
 
 // Launches a kernel of one CTA per set, at most as many CTAs as are resident
-// at once with `smem` bytes of dynamic shared memory.
+// at once with `smem` bytes of dynamic shared memory (at most `smem_max`). The
+// kernel's limit is state of the process that other threads' builds share, so
+// it is always set to the same value, whatever this call needs.
 template <typename... Params, typename... Args>
-cudaError_t launch_sets(void (*kernel)(Params...), int64_t sets, size_t smem, int num_sms, cudaStream_t st,
-                        Args... args) {
+cudaError_t launch_sets(void (*kernel)(Params...), int64_t sets, size_t smem, size_t smem_max, int num_sms,
+                        cudaStream_t st, Args... args) {
     int per_sm = 0;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess ||
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_max))) !=
+            cudaSuccess ||
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSetThreads, smem)) != cudaSuccess)
         return e;
     const int64_t grid = std::min<int64_t>(sets, int64_t(num_sms) * std::max(per_sm, 1));
@@ -812,10 +815,10 @@ cudaError_t DeviceBuild::stage(const uint8_t *h_bytes, const int64_t *h_off, con
     }
     if (e != cudaSuccess) return e;
     if (small_ &&
-        ((e = launch_sets(k_b_set_sort, M, sort_smem(smax_), num_sms, st, static_cast<const uint8_t *>(s_->bytes),
-                          static_cast<const int64_t *>(s_->off), static_cast<const int32_t *>(s_->set_off), M, smax_,
-                          static_cast<const int32_t *>(s_->flags), s_->order, s_->count, s_->n_chars)) !=
-             cudaSuccess ||
+        ((e = launch_sets(k_b_set_sort, M, sort_smem(smax_), sort_smem(kSetMaxStrings), num_sms, st,
+                          static_cast<const uint8_t *>(s_->bytes), static_cast<const int64_t *>(s_->off),
+                          static_cast<const int32_t *>(s_->set_off), M, smax_, static_cast<const int32_t *>(s_->flags),
+                          s_->order, s_->count, s_->n_chars)) != cudaSuccess ||
          (e = launch_pdl(k_b_set_scan, 1, kBThreads, st, M, static_cast<const int32_t *>(s_->count), s_->roots,
                          s_->total)) != cudaSuccess))
         return e;
@@ -923,7 +926,8 @@ cudaError_t DeviceBuild::emit(int32_t *parent, uint8_t *label, uint8_t *terminal
     if (small_) {
         // a few sets: their depths over several CTAs each, up to four CTAs an SM
         const int32_t parts = int32_t(std::min<int64_t>(8, std::max<int64_t>(1, 4 * int64_t(num_sms) / M_)));
-        return launch_sets(k_b_set_nodes, int64_t(M_) * parts, nodes_smem(smax_, D_), num_sms, stream_,
+        return launch_sets(k_b_set_nodes, int64_t(M_) * parts, nodes_smem(smax_, D_),
+                           nodes_smem(kSetMaxStrings, kDeviceBuildMaxDepth), num_sms, stream_,
                            static_cast<const uint8_t *>(s_->bytes), static_cast<const int64_t *>(s_->off),
                            static_cast<const int32_t *>(s_->set_off), M_, smax_, D_, parts,
                            static_cast<const uint2 *>(s_->order), static_cast<const int32_t *>(s_->roots), parent,
