@@ -95,6 +95,24 @@ void pool_free(void *p) {
     cudaGetLastError();
 }
 
+// The calling thread in the relaxed capture mode: in the default one event
+// queries and stream-ordered frees are refused on any stream while some thread
+// of the process captures one, and that capture then fails.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Whether the work before an event has run. An error is no answer, so it
+// counts as not done.
+bool event_done(cudaEvent_t ev) {
+    RelaxedCapture relaxed;
+    const cudaError_t q = cudaEventQuery(ev);
+    if (q != cudaSuccess) cudaGetLastError();
+    return q == cudaSuccess;
+}
+
 std::mutex g_vocab_mu;
 // Most recent last. Never destroyed, so no device memory is freed during
 // static destruction at process exit (the CUDA runtime may be gone by then).
@@ -948,9 +966,7 @@ static void *take_spare_block(int dev, size_t bytes) {
         SpareBlock &b = g_spare[i];
         if (b.dev != dev || b.bytes < bytes || b.bytes > 2 * bytes) continue;
         if (b.ready) {
-            const cudaError_t q = cudaEventQuery(b.ready);
-            if (q == cudaErrorNotReady) continue;
-            cudaGetLastError();
+            if (!event_done(b.ready)) continue;
             cudaEventDestroy(b.ready);
         }
         void *p = b.p;
@@ -977,9 +993,8 @@ static void give_spare_block(int dev, void *p, size_t bytes, cudaEvent_t ready, 
             if (b.dev != dev) continue;
             held++;
             if (b.bytes >= (least ? least->bytes : bytes)) continue;
-            if (!b.ready || cudaEventQuery(b.ready) == cudaSuccess) least = &b;
+            if (!b.ready || event_done(b.ready)) least = &b;
         }
-        cudaGetLastError();
         if (held < kSpareListBlocks) {
             g_spare.push_back(out);
             return;
@@ -1591,12 +1606,10 @@ static void sweep_retired() {
         std::lock_guard<std::mutex> lk(g_retired_mu);
         size_t keep = 0;
         for (size_t i = 0; i < g_retired.size(); i++) {
-            const cudaError_t q = cudaEventQuery(g_retired[i].first);
-            if (q == cudaErrorNotReady) {
+            if (!event_done(g_retired[i].first)) {
                 g_retired[keep++] = g_retired[i];
                 continue;
             }
-            cudaGetLastError();
             cudaEventDestroy(g_retired[i].first);
             done.push_back(g_retired[i].second);
         }
@@ -1615,6 +1628,7 @@ static void retire_handle(trie_t h, cudaEvent_t ev) {
 
 int trie_destroy_async(trie_t h, cudaStream_t stream) {
     if (!h) return TRIE_OK;
+    RelaxedCapture relaxed;
     int rc = TRIE_OK;
     auto free_on = [&](void *p) {
         if (!p) return;
