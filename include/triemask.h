@@ -62,7 +62,10 @@
  * and is asynchronous with respect to the host. Concurrent trie_advance /
  * trie_apply_mask calls on one handle are safe (they only read the trie and
  * the mask); trie_compile_masks and trie_destroy must not race with other
- * calls on the same handle.
+ * calls on the same handle. A call on a stream that is being captured makes
+ * what the handle keeps (its memory, the trie's upload) at once and outside
+ * the graph, which holds the kernels only; the vocabulary must be known to the
+ * library by then (trie_vocab_create, or an earlier call).
  */
 #ifndef TRIEMASK_H
 #define TRIEMASK_H

@@ -73,11 +73,58 @@ struct Layout {
 // on the device, so an allocation carries no stream dependency.
 constexpr uint64_t kPoolKeepBytes = uint64_t(8) << 30;
 
+// The calling thread in the relaxed capture mode: in the default one event
+// queries and stream-ordered frees are refused on any stream while some thread
+// of the process captures one, and that capture then fails.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Whether a graph capture is under way on the stream.
+bool is_capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) cudaGetLastError();
+    return st == cudaStreamCaptureStatusActive;
+}
+
+// What a call on a captured stream sets up for the handle's later calls too
+// (its memory, the trie's upload) is done at once on a stream of its own: as
+// part of the graph it would be there only once the graph has run.
+class OutsideCapture {
+public:
+    OutsideCapture() { error_ = cudaStreamCreateWithFlags(&side_, cudaStreamNonBlocking); }
+    ~OutsideCapture() {
+        if (side_) cudaStreamDestroy(side_);
+    }
+    OutsideCapture(const OutsideCapture &) = delete;
+    OutsideCapture &operator=(const OutsideCapture &) = delete;
+    cudaStream_t stream() const { return side_; }
+    cudaError_t error() const { return error_; }
+    cudaError_t finish() { return cudaStreamSynchronize(side_); }
+
+private:
+    RelaxedCapture relaxed_;
+    cudaStream_t side_ = nullptr;
+    cudaError_t error_;
+};
+
+cudaError_t alloc_outside_capture(void **out, size_t bytes, cudaMemPool_t pool) {
+    OutsideCapture side;
+    if (side.error() != cudaSuccess) return side.error();
+    const cudaError_t e = cudaMallocFromPoolAsync(out, bytes, pool, side.stream());
+    const cudaError_t done = side.finish();
+    return e != cudaSuccess ? e : done;
+}
+
 int pool_alloc(int dev, size_t bytes, cudaStream_t stream, void **out, const char *what) {
     *out = nullptr;
     cudaMemPool_t pool = tmk::device_pool(dev);
     if (!pool) return fail(TRIE_ECUDA, std::string("creating the device memory pool for ") + what);
-    cudaError_t e = cudaMallocFromPoolAsync(out, std::max<size_t>(bytes, 1), pool, stream);
+    bytes = std::max<size_t>(bytes, 1);
+    cudaError_t e = is_capturing(stream) ? alloc_outside_capture(out, bytes, pool)
+                                         : cudaMallocFromPoolAsync(out, bytes, pool, stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *out = nullptr;
@@ -94,15 +141,6 @@ void pool_free(void *p) {
     cudaFreeAsync(p, 0);
     cudaGetLastError();
 }
-
-// The calling thread in the relaxed capture mode: in the default one event
-// queries and stream-ordered frees are refused on any stream while some thread
-// of the process captures one, and that capture then fails.
-struct RelaxedCapture {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
 
 // Whether the work before an event has run. An error is no answer, so it
 // counts as not done.
@@ -202,9 +240,6 @@ int get_vocab(const uint8_t *vb, const int64_t *vo, int32_t V, int dev,
     return TRIE_OK;
 }
 
-// Uploads the trie on first use, ordered on `stream` (the copies read the
-// handle's own host arrays, which outlive them); the handle is bound to that
-// device.
 // The segment summary of the dense mask (bit g of row r set iff the row allows
 // a token of the 1,024-token segment g), which lets the apply skip reading
 // the mask words of empty segments; none when it would exceed 256 MB, and
@@ -289,6 +324,7 @@ int alloc_device_trie(trie_t h, int dev, size_t n, cudaStream_t stream, bool sin
     h->dev.first_child = reinterpret_cast<int32_t *>(b + o_fc);
     h->dev.child_bits = reinterpret_cast<uint32_t *>(b + o_bits);
     if (single) tables.place(&h->dev, b);
+    h->dev.tables_ready = single;  // once finish_device_trie has launched their kernel
     h->dev.trans = single ? reinterpret_cast<ulonglong2 *>(b + o_trans) : nullptr;
     h->dev.trans_mask = single ? uint32_t(trans_slots - 1) : 0u;
     return TRIE_OK;
@@ -310,38 +346,29 @@ int finish_device_trie(trie_t h, int dev, cudaStream_t stream, const ClearRange 
 
 // A forest's compile tables, on the first call that reads them (81 B and 16
 // dependent loads per node: 80 us and 386 MB for 4.77 M nodes that a forest
-// compiled to lists never uses). The caller must be a call that does not run
-// beside others on the handle.
+// compiled to lists never uses). A graph that captures such a call fills them
+// whenever it runs; as it may never run, the next call outside fills them too.
+// The caller must be a call that does not run beside others on the handle.
 int ensure_tables(trie_t h, int dev, cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(h->mu);
-    if (h->dev.window) return TRIE_OK;
-    Layout L;
-    const TableLayout tables(L, size_t(h->host.n));
-    void *base = nullptr;
-    const int rc = pool_alloc(dev, L.total, stream, &base, "the trie's compile tables");
-    if (rc != TRIE_OK) return rc;
-    tables.place(&h->dev, static_cast<char *>(base));
-    const cudaError_t e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
-    if (e != cudaSuccess) {
-        h->dev.window = nullptr;
-        pool_free(base);
-        return fail_cuda(e, "building the trie's compile tables");
+    if (h->dev.tables_ready) return TRIE_OK;
+    if (!h->dev.window) {
+        Layout L;
+        const TableLayout tables(L, size_t(h->host.n));
+        const int rc = pool_alloc(dev, L.total, stream, &h->dev.tables_base, "the trie's compile tables");
+        if (rc != TRIE_OK) return rc;
+        tables.place(&h->dev, static_cast<char *>(h->dev.tables_base));
     }
-    h->dev.tables_base = base;
+    const cudaError_t e = tmk::launch_trie_tables(h->dev, h->host.n, num_sms(dev), stream);
+    if (e != cudaSuccess) return fail_cuda(e, "building the trie's compile tables");
+    h->dev.tables_ready = !is_capturing(stream);
     return TRIE_OK;
 }
 
 bool host_memory_direct(int dev);
 
-// dense_words: as in alloc_device_trie.
-int ensure_device_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_words = 0) {
-    std::lock_guard<std::mutex> lk(h->mu);
-    if (h->dev.base) {
-        if (h->dev.device != dev)
-            return fail(TRIE_EINVAL, "handle was uploaded to device " + std::to_string(h->dev.device) +
-                                         ", called on device " + std::to_string(dev));
-        return TRIE_OK;
-    }
+// Uploads the trie (h->mu held; dense_words as in alloc_device_trie).
+int upload_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_words) {
     const tmk::HostTrie &t = h->host;
     const size_t n = size_t(t.n);
     // a transition table for a single trie; a forest's per-request sets are
@@ -377,6 +404,27 @@ int ensure_device_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_wor
         }
     }
     return finish_device_trie(h, dev, stream, clear);
+}
+
+// Uploads the trie on first use, ordered on `stream` (the copies read the
+// handle's own host arrays, which outlive them); the handle is bound to that
+// device.
+int ensure_device_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_words = 0) {
+    std::lock_guard<std::mutex> lk(h->mu);
+    if (h->dev.base) {
+        if (h->dev.device != dev)
+            return fail(TRIE_EINVAL, "handle was uploaded to device " + std::to_string(h->dev.device) +
+                                         ", called on device " + std::to_string(dev));
+        return TRIE_OK;
+    }
+    if (is_capturing(stream)) {
+        OutsideCapture side;
+        if (side.error() != cudaSuccess) return fail_cuda(side.error(), "creating a stream for the trie's upload");
+        const int rc = upload_trie(h, dev, side.stream(), dense_words);
+        const cudaError_t e = side.finish();
+        return rc != TRIE_OK || e == cudaSuccess ? rc : fail_cuda(e, "uploading the trie");
+    }
+    return upload_trie(h, dev, stream, dense_words);
 }
 
 // The transition table holds transitions of one vocabulary: when a compile

@@ -253,6 +253,7 @@ struct DevTrie {
     ulonglong2 *window = nullptr;    // [n]
     uint8_t *depth16 = nullptr;      // [n]
     int4 *anc = nullptr;             // [n * 4]
+    bool tables_ready = false;       // a kernel that fills them has been launched (not only captured)
     ulonglong2 *trans = nullptr;     // transition table {(row << 32 | token) + 1, end node}
     uint32_t trans_mask = 0;         // slots - 1
     bool trans_clean = false;        // the table was cleared at the upload and not used since

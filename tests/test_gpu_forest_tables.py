@@ -67,3 +67,45 @@ def test_lazy_setup_behind_an_upload_on_another_stream():
     m = T.trie_lazy_rows(h, torch.arange(h.num_nodes, dtype=torch.int32, device="cuda"), V)
     assert np.array_equal(m.cpu().numpy().view(np.uint32), want)
     h.destroy()
+
+
+@pytest.mark.parametrize("build", ["single", "host", "device"])
+@pytest.mark.parametrize("uploaded", [False, True])
+def test_first_compile_captured(build, uploaded):
+    """A handle's first dense compile (and, if nothing did it before, its upload)
+    is captured, and the graph has not run yet when calls outside it need the
+    same arrays, tables and buffers."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    oracle.build()
+    strings, toks = random_case(91)
+    sets = [strings] if build == "single" else [strings, strings[:3]]
+    sb, so = W.pack([x for s in sets for x in s])
+    si = np.cumsum([0] + [len(s) for s in sets]).astype(np.int32)
+    vb, vo = W.pack(toks)
+    V = len(toks)
+    voc = T.trie_vocab_create(vb, vo, V)
+    h = T.trie_build(sb, so) if build == "single" else \
+        (T.trie_build_many_device if build == "device" else T.trie_build_many)(sb, so, si)
+    ov = oracle.Vocab(vb, vo)
+    want = np.concatenate([oracle.mask_all(oracle.Trie(*W.pack(s)), ov) for s in sets])
+    if uploaded:
+        T.trie_compile_lists_vocab(h, voc)
+    first, second = torch.empty((2, h.num_nodes, T.mask_words(V)), dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        T.trie_compile_masks_vocab(h, voc, first)
+    T.trie_compile_masks_vocab(h, voc, second)
+    assert np.array_equal(second.cpu().numpy().view(np.uint32), want)
+    T.trie_lazy_init(h, vb, vo, V, cache_rows=0, max_batch=h.num_nodes)
+    m = T.trie_lazy_rows(h, torch.arange(h.num_nodes, dtype=torch.int32, device="cuda"), V)
+    assert np.array_equal(m.cpu().numpy().view(np.uint32), want)
+    for _ in range(2):
+        first.fill_(-1)
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(first.cpu().numpy().view(np.uint32), want)
+    del g
+    h.destroy()
