@@ -28,7 +28,7 @@ namespace {
 
 constexpr int kBThreads = 256;
 // Forests whose sets all hold at most this many strings are sorted, one CTA
-// per set (38 B of shared memory a string). 256 sets of 300-2,000 names: 54 us
+// per set (42 B of shared memory a string). 256 sets of 300-2,000 names: 54 us
 // to sort and 30 us to write the nodes, against 178 and 12 us by one CTA per
 // set inserting level by level (seven barriers for each of ~32 levels), and
 // 630 us by the level kernels over all sets.
@@ -386,11 +386,11 @@ __device__ __forceinline__ int32_t set_excl_scan(int32_t v, int32_t *ws, int32_t
     return before + x - v;
 }
 
-// The first min(len, kSetKeyBytes) bytes at p as big-endian words (zeros
-// after them), by the aligned 8-byte words that hold them (all inside the
-// staged image: only words with a byte of the string are read).
-__device__ __forceinline__ void load_key(const uint8_t *p, int32_t len, uint64_t (&w)[kSetKeyWords]) {
-    const int32_t n = len < kSetKeyBytes ? len : kSetKeyBytes;
+// The first min(len, most) bytes at p as big-endian words (zeros after them),
+// most <= kSetKeyBytes, by the aligned 8-byte words that hold them (all inside
+// the staged image: only words with a byte of the string are read).
+__device__ __forceinline__ void load_key(const uint8_t *p, int32_t len, int32_t most, uint64_t (&w)[kSetKeyWords]) {
+    const int32_t n = len < most ? len : most;
     const uint32_t mis = uint32_t(reinterpret_cast<uintptr_t>(p)) & 7u;
     const uint64_t *q = reinterpret_cast<const uint64_t *>(p - mis);
     uint64_t raw[kSetKeyWords + 1];
@@ -410,62 +410,137 @@ __device__ __forceinline__ void load_key(const uint8_t *p, int32_t len, uint64_t
 
 // The strings of one set in shared memory: the key of string j in two halves
 // of 16 bytes (key[j], key[cap + j]: one load compares 16 bytes, and names of
-// one stem agree in their first 8), its length, and its place in the image.
+// one stem agree in their first 8) and its length. The key holds the string's
+// bytes base .. limit - 1, at first the first kSetKeyBytes. Strings that agree
+// in those and go on are sorted again by the bytes after them; their keys then
+// begin with the number of the group of such neighbours (kGroupBytes of it).
+constexpr int kGroupBytes = 2;
+
 struct SetStrings {
-    const ulonglong2 *key;
+    ulonglong2 *key;
     int32_t cap;
-    const uint16_t *len;
-    const uint8_t *bytes;
-    const int64_t *off;  // of the set's first string
-    int64_t off0;
+    uint16_t *len;
+    int32_t base;
+    int32_t limit;
 
-    __device__ __forceinline__ uint32_t byte(int32_t j, int32_t k) const { return bytes[off[j] - off0 + k]; }
-
-    // Bytes that strings a and b have in common from their start.
+    // What strings a and b of one group have in common from their start, or -1
+    // where that is more than their keys show.
     __device__ __forceinline__ int32_t common(int32_t a, int32_t b) const {
         const int32_t n = min(int32_t(len[a]), int32_t(len[b]));
+        const int32_t from = base ? base - kGroupBytes : 0;
 #pragma unroll
         for (int h = 0; h < kSetKeyWords / 2; h++) {
             const ulonglong2 x = key[h * cap + a], y = key[h * cap + b];
-            if (x.x != y.x) return min(n, 16 * h + (__clzll(static_cast<long long>(x.x ^ y.x)) >> 3));
-            if (x.y != y.y) return min(n, 16 * h + 8 + (__clzll(static_cast<long long>(x.y ^ y.y)) >> 3));
+            if (x.x != y.x) return min(n, from + 16 * h + (__clzll(static_cast<long long>(x.x ^ y.x)) >> 3));
+            if (x.y != y.y) return min(n, from + 16 * h + 8 + (__clzll(static_cast<long long>(x.y ^ y.y)) >> 3));
         }
-        int32_t k = min(n, kSetKeyBytes);
-        while (k < n && byte(a, k) == byte(b, k)) k++;
-        return k;
+        return n <= limit ? n : -1;
     }
 
-    // Whether a sorts before b; a0 and b0 are the first halves of their keys.
+    // Whether a sorts before b by their keys; a0 and b0 are the first halves.
     __device__ __forceinline__ bool before(int32_t a, ulonglong2 a0, int32_t b, ulonglong2 b0) const {
         if (a0.x != b0.x) return a0.x < b0.x;
         if (a0.y != b0.y) return a0.y < b0.y;
         const ulonglong2 a1 = key[cap + a], b1 = key[cap + b];
         if (a1.x != b1.x) return a1.x < b1.x;
         if (a1.y != b1.y) return a1.y < b1.y;
-        const int32_t la = len[a], lb = len[b], n = min(la, lb);
-        for (int32_t k = kSetKeyBytes; k < n; k++) {
-            const uint32_t x = byte(a, k), y = byte(b, k);
-            if (x != y) return x < y;
-        }
-        return la < lb;  // a prefix, then what it is a prefix of
+        const int32_t la = len[a];
+        return la <= limit && la < int32_t(len[b]);  // a prefix, then what it is a prefix of
     }
 };
 
-// Sorts the strings of every set and gives their order: order[i] (i counted
-// from the set's first string) = {lcp | len << 16, string within the set},
-// the set's node count, and the characters of its distinct strings. Merge sort
-// of 2-byte indices: every thread sorts kSortPer strings, then in each round
-// finds by a search along its output's diagonal where its next kSortPer
-// outputs begin in the two runs, and merges them. Bound by the chain of
-// shared-memory loads of the searches: about 3 us a round at 1,203 strings, 31
-// us in all. (Measured slower: every element searched for by itself in the
-// neighbouring run, four side by side, 68 us for the 256 sets; 8-byte words of
-// the key compared one load after the other, and keys of 32 contiguous bytes,
-// whose first halves share half of the banks, 65 us.) Does nothing when the
-// staging found bad offsets or a string longer than the build takes (flags).
+// Sorts the n strings listed in src by their keys, with dst for the rounds;
+// the result is in src. Merge sort of 2-byte indices: every thread sorts
+// kSortPer strings, then in each round finds by a search along its output's
+// diagonal where its next kSortPer outputs begin in the two runs, and merges
+// them. Ends with a barrier.
 constexpr int kSortPer = 4;
 
-__global__ void __launch_bounds__(kSetThreads) k_b_set_sort(const uint8_t *__restrict__ bytes,
+__device__ __forceinline__ void sort_strings(const SetStrings &str, uint16_t *&src, uint16_t *&dst, int32_t n) {
+    const int tid = threadIdx.x;
+    const ulonglong2 *const key = str.key;
+    for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
+        int32_t x[kSortPer];
+        ulonglong2 x0[kSortPer];
+        const int32_t m = min(kSortPer, n - o);
+#pragma unroll
+        for (int e = 0; e < kSortPer; e++) {
+            x[e] = src[e < m ? o + e : o];
+            x0[e] = key[x[e]];
+        }
+#pragma unroll
+        for (int r = 1; r < kSortPer; r++)
+#pragma unroll
+            for (int e = r; e > 0; e--)
+                if (r < m && str.before(x[e], x0[e], x[e - 1], x0[e - 1])) {
+                    const int32_t y = x[e];
+                    const ulonglong2 y0 = x0[e];
+                    x[e] = x[e - 1], x0[e] = x0[e - 1];
+                    x[e - 1] = y, x0[e - 1] = y0;
+                }
+#pragma unroll
+        for (int e = 0; e < kSortPer; e++)
+            if (e < m) src[o + e] = uint16_t(x[e]);
+    }
+    __syncthreads();
+    for (int32_t w = kSortPer; w < n; w <<= 1) {
+        for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
+            const int32_t first = o & ~(2 * w - 1), diag = o - first;
+            const int32_t na = min(w, n - first), nb = max(0, min(w, n - first - w));
+            const uint16_t *A = src + first, *B = A + w;
+            int32_t lo = max(0, diag - nb), hi = min(diag, na);
+            while (lo < hi) {  // the entries of A among the first diag outputs
+                const int32_t mid = (lo + hi) >> 1;
+                const int32_t x = A[mid], y = B[diag - 1 - mid];
+                if (str.before(y, key[y], x, key[x])) hi = mid;
+                else lo = mid + 1;
+            }
+            int32_t ia = lo, ib = diag - lo;
+            int32_t x = ia < na ? int32_t(A[ia]) : 0, y = ib < nb ? int32_t(B[ib]) : 0;
+            ulonglong2 x0 = key[x], y0 = key[y];
+#pragma unroll
+            for (int e = 0; e < kSortPer; e++) {
+                if (o + e >= n) break;
+                const bool from_b = ib < nb && (ia >= na || str.before(y, y0, x, x0));
+                dst[o + e] = uint16_t(from_b ? y : x);
+                if (from_b) {
+                    ib++;
+                    if (ib < nb) y = B[ib], y0 = key[y];
+                } else {
+                    ia++;
+                    if (ia < na) x = A[ia], x0 = key[x];
+                }
+            }
+        }
+        __syncthreads();
+        uint16_t *const t = src;
+        src = dst;
+        dst = t;
+    }
+}
+
+// Sorts the strings of every set and gives their order: order[i] (i counted
+// from the set's first string) = {lcp | len << 16, string within the set},
+// the set's node count, and the characters of its distinct strings. The
+// strings are sorted by their first kSetKeyBytes bytes; neighbours that agree
+// in them and go on form groups, whose strings alone get the next bytes as
+// keys, and are sorted again where those are not in order yet, until no two
+// neighbours agree in all bytes looked at. So a root that all strings share is
+// passed at a load and a comparison per kSetKeyBytes - kGroupBytes bytes (16
+// sets of 1,200 strings of 24 bytes behind a root of 512: the build takes 0.27
+// ms, 0.09 ms without the root; 29 ms where every comparison of the sort went
+// through the root byte by byte). Three CTAs an SM, at 40 registers: at 64 a
+// build of 2,000 sets of 100 strings takes 254 us, 231 us so.
+// Bound by the chain of shared-memory loads of the merge sort's searches: about
+// 3 us a round at 1,203 strings, 31 us in all. (Measured slower: every element
+// searched for by itself in the neighbouring run, four side by side, 68 us for
+// the 256 sets; 8-byte words of the key compared one load after the other, and
+// keys of 32 contiguous bytes, whose first halves share half of the banks, 65
+// us.) Does nothing when the staging found bad offsets or a string longer than
+// the build takes (flags).
+static_assert(kSetMaxStrings / kSetThreads <= 32, "a thread's places in the order have a bit each");
+
+__global__ void __launch_bounds__(kSetThreads, 3) k_b_set_sort(const uint8_t *__restrict__ bytes,
                                                             const int64_t *__restrict__ off,
                                                             const int32_t *__restrict__ set_off, int32_t M,
                                                             int32_t cap, const int32_t *__restrict__ flags,
@@ -474,8 +549,10 @@ __global__ void __launch_bounds__(kSetThreads) k_b_set_sort(const uint8_t *__res
     extern __shared__ uint4 dyn[];
     ulonglong2 *key = reinterpret_cast<ulonglong2 *>(dyn);
     uint16_t *len = reinterpret_cast<uint16_t *>(key + 2 * size_t(cap));
-    uint16_t *const ids = len + cap;  // [2 * cap]: the order before and after a round
+    uint16_t *const pos = len + cap, *const lcp = pos + cap;  // the order, and what each string shares with the one before
+    uint16_t *list = lcp + cap, *buf = list + cap;            // the strings to sort, and the sort's other side
     __shared__ int32_t ws[kSetThreads / 32];
+    __shared__ uint8_t edge[kSetThreads + 1];
     pdl_launch_dependents();
     pdl_wait();
     if (flags[0] != 0 || flags[1] > kDeviceBuildMaxDepth) return;
@@ -487,79 +564,76 @@ __global__ void __launch_bounds__(kSetThreads) k_b_set_sort(const uint8_t *__res
             const int64_t a = off[i0 + j];
             const int32_t l = int32_t(off[i0 + j + 1] - a);
             uint64_t w[kSetKeyWords];
-            load_key(bytes + (a - off0), l, w);
+            load_key(bytes + (a - off0), l, kSetKeyBytes, w);
             key[j] = make_ulonglong2(w[0], w[1]);
             key[cap + j] = make_ulonglong2(w[2], w[3]);
             len[j] = uint16_t(l);
+            list[j] = uint16_t(j);
         }
         __syncthreads();
-        const SetStrings str{key, cap, len, bytes, off + i0, off0};
-        uint16_t *src = ids, *dst = ids + cap;
-        for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
-            int32_t x[kSortPer];
-            ulonglong2 x0[kSortPer];
-            const int32_t m = min(kSortPer, n - o);
-#pragma unroll
-            for (int e = 0; e < kSortPer; e++) {
-                x[e] = e < m ? o + e : o;
-                x0[e] = key[x[e]];
+        SetStrings str{key, cap, len, 0, kSetKeyBytes};
+        // this thread's places in the order, r0 .. r1 - 1. Bit k of tied: the
+        // string at place r0 + k is in the list; of joined: it agrees with the
+        // one before it in all bytes looked at.
+        const int32_t per = (n + kSetThreads - 1) / kSetThreads;
+        const int32_t r0 = min(tid * per, n), r1 = min(r0 + per, n);
+        uint32_t tied = (1u << (r1 - r0)) - 1u;
+        uint32_t joined = r0 ? tied : tied & ~1u;
+        int32_t listed = n, at0 = r0;  // strings in the list; this thread's first
+        bool in_order = false;
+        if (r0 == 0 && n > 0) lcp[0] = 0;
+        while (true) {
+            if (!in_order) {
+                sort_strings(str, list, buf, listed);
+                for (int32_t k = 0, at = at0; k < r1 - r0; k++)
+                    if ((tied >> k) & 1u) pos[r0 + k] = list[at++];
+                __syncthreads();
             }
-#pragma unroll
-            for (int r = 1; r < kSortPer; r++)
-#pragma unroll
-                for (int e = r; e > 0; e--)
-                    if (r < m && str.before(x[e], x0[e], x[e - 1], x0[e - 1])) {
-                        const int32_t y = x[e];
-                        const ulonglong2 y0 = x0[e];
-                        x[e] = x[e - 1], x0[e] = x0[e - 1];
-                        x[e - 1] = y, x0[e - 1] = y0;
-                    }
-#pragma unroll
-            for (int e = 0; e < kSortPer; e++)
-                if (e < m) src[o + e] = uint16_t(x[e]);
-        }
-        __syncthreads();
-        for (int32_t w = kSortPer; w < n; w <<= 1) {
-            for (int32_t o = kSortPer * tid; o < n; o += kSortPer * kSetThreads) {
-                const int32_t first = o & ~(2 * w - 1), diag = o - first;
-                const int32_t na = min(w, n - first), nb = max(0, min(w, n - first - w));
-                const uint16_t *A = src + first, *B = A + w;
-                int32_t lo = max(0, diag - nb), hi = min(diag, na);
-                while (lo < hi) {  // the entries of A among the first diag outputs
-                    const int32_t mid = (lo + hi) >> 1;
-                    const int32_t x = A[mid], y = B[diag - 1 - mid];
-                    if (str.before(y, key[y], x, key[x])) hi = mid;
-                    else lo = mid + 1;
-                }
-                int32_t ia = lo, ib = diag - lo;
-                int32_t x = ia < na ? int32_t(A[ia]) : 0, y = ib < nb ? int32_t(B[ib]) : 0;
-                ulonglong2 x0 = key[x], y0 = key[y];
-#pragma unroll
-                for (int e = 0; e < kSortPer; e++) {
-                    if (o + e >= n) break;
-                    const bool from_b = ib < nb && (ia >= na || str.before(y, y0, x, x0));
-                    dst[o + e] = uint16_t(from_b ? y : x);
-                    if (from_b) {
-                        ib++;
-                        if (ib < nb) y = B[ib], y0 = key[y];
-                    } else {
-                        ia++;
-                        if (ia < na) x = A[ia], x0 = key[x];
-                    }
-                }
+            for (int32_t k = 0; k < r1 - r0; k++) {
+                if (!((joined >> k) & 1u)) continue;
+                const int32_t c = str.common(pos[r0 + k - 1], pos[r0 + k]);
+                if (c < 0) continue;
+                lcp[r0 + k] = uint16_t(c);
+                joined &= ~(1u << k);
+            }
+            if (tid == 0) edge[kSetThreads] = 0;
+            edge[tid] = uint8_t(joined & 1u);
+            if (!__syncthreads_or(joined != 0u)) break;
+            tied = joined | (joined >> 1);  // joined, or the string after it is
+            if (r1 < n && edge[tid + 1]) tied |= 1u << (r1 - r0 - 1);
+            const uint32_t heads = tied & ~joined;
+            str.base = str.limit;
+            str.limit += kSetKeyBytes - kGroupBytes;
+            const int32_t before = set_excl_scan(__popc(tied) | (__popc(heads) << 16), ws, &listed);
+            listed &= 0xFFFF;
+            at0 = before & 0xFFFF;
+            int32_t group = before >> 16;
+            for (int32_t k = 0, at = at0; k < r1 - r0; k++) {
+                if (!((tied >> k) & 1u)) continue;
+                group += int32_t((heads >> k) & 1u);
+                const int32_t b = pos[r0 + k];
+                uint64_t w[kSetKeyWords];
+                load_key(bytes + (off[i0 + b] - off0) + str.base, int32_t(len[b]) - str.base,
+                         kSetKeyBytes - kGroupBytes, w);
+                key[b] = make_ulonglong2((w[0] >> 16) | (uint64_t(group) << 48), (w[1] >> 16) | (w[0] << 48));
+                key[cap + b] = make_ulonglong2((w[2] >> 16) | (w[1] << 48), (w[3] >> 16) | (w[2] << 48));
+                list[at++] = uint16_t(b);
             }
             __syncthreads();
-            uint16_t *const t = src;
-            src = dst;
-            dst = t;
+            in_order = true;
+            for (int32_t k = 0; k < r1 - r0; k++) {
+                if (!((joined >> k) & 1u)) continue;
+                const int32_t x = pos[r0 + k], y = pos[r0 + k - 1];
+                in_order = in_order && !str.before(x, key[x], y, key[y]);
+            }
+            in_order = !__syncthreads_or(!in_order);
         }
         int32_t nodes = 0, my_chars = 0;
         for (int32_t i = tid; i < n; i += kSetThreads) {
-            const int32_t b = src[i], l = len[b];
-            const int32_t lcp = i > 0 ? str.common(src[i - 1], b) : 0;
-            order[i0 + i] = make_uint2(uint32_t(lcp) | (uint32_t(l) << 16), uint32_t(b));
-            nodes += l - lcp;
-            if (i == 0 || lcp < l) my_chars += l;  // not a repetition of the string before it
+            const int32_t b = pos[i], l = len[b], c = lcp[i];
+            order[i0 + i] = make_uint2(uint32_t(c) | (uint32_t(l) << 16), uint32_t(b));
+            nodes += l - c;
+            if (i == 0 || c < l) my_chars += l;  // not a repetition of the string before it
         }
         int32_t total, total_chars;
         set_excl_scan(nodes, ws, &total);
@@ -740,7 +814,7 @@ struct Carver {
 // 0, characters (8 bytes)}, then the roots.
 constexpr size_t kHeadRoots = 24;
 
-size_t sort_smem(int32_t cap) { return size_t(cap) * (kSetKeyBytes + 3 * sizeof(uint16_t)); }
+size_t sort_smem(int32_t cap) { return size_t(cap) * (kSetKeyBytes + 5 * sizeof(uint16_t)); }
 size_t nodes_smem(int32_t cap, int32_t D) {
     return size_t(cap) * sizeof(uint2) + sizeof(int32_t) * (size_t(D) + 2);
 }
