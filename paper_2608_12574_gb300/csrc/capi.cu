@@ -1298,6 +1298,47 @@ int64_t trie_num_valid(trie_t h) {
     return L.n_valid;
 }
 
+// The tokens out of the {token, end node} entries into any memory that a copy
+// takes. A kernel gathers them: straight into the handle's device, managed or
+// pinned memory, else into scratch that one copy moves on. (A strided copy, a
+// row of 4 bytes an entry, took 4.9 ms for 14.3 M entries into pinned memory.)
+// The strided copy stays for what is left: a stream of another device, where
+// the kernel cannot run, other memory under capture, and no scratch.
+static cudaError_t copy_tokens(trie_t h, int32_t *tokens, cudaStream_t stream) {
+    const tmk::DevLists &L = h->lists;
+    const int dev = h->dev.device;
+    const int64_t n = L.n_valid;
+    int stream_dev = -1;
+    if (cudaGetDevice(&stream_dev) != cudaSuccess) cudaGetLastError();
+    // (the default streams are the current device's; a captured stream may not be asked)
+    const bool named = stream && stream != cudaStreamLegacy && stream != cudaStreamPerThread;
+    if (named && !is_capturing(stream)) {
+        RelaxedCapture relaxed;
+        if (cudaStreamGetDevice(stream, &stream_dev) != cudaSuccess) cudaGetLastError();
+    }
+    DeviceGuard g(dev);
+    const size_t bytes = sizeof(int32_t) * size_t(n);
+    if (stream_dev == dev) {
+        cudaPointerAttributes at = {};
+        if (cudaPointerGetAttributes(&at, tokens) != cudaSuccess) cudaGetLastError();
+        const bool near = (at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged ||
+                          at.type == cudaMemoryTypeHost;
+        if (near && at.devicePointer && (reinterpret_cast<uintptr_t>(at.devicePointer) & 3u) == 0)
+            return tmk::launch_copy_tokens(L, n, static_cast<int32_t *>(at.devicePointer), num_sms(dev), stream);
+        void *tmp = nullptr;
+        cudaMemPool_t pool = is_capturing(stream) ? nullptr : tmk::device_pool(dev);
+        if (pool && cudaMallocFromPoolAsync(&tmp, bytes, pool, stream) == cudaSuccess) {
+            cudaError_t e = tmk::launch_copy_tokens(L, n, static_cast<int32_t *>(tmp), num_sms(dev), stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(tokens, tmp, bytes, cudaMemcpyDeviceToDevice, stream);
+            const cudaError_t freed = cudaFreeAsync(tmp, stream);
+            return e != cudaSuccess ? e : freed;
+        }
+        cudaGetLastError();
+    }
+    return cudaMemcpy2DAsync(tokens, sizeof(int32_t), L.entries, sizeof(int2), sizeof(int32_t), size_t(n),
+                             cudaMemcpyDeviceToDevice, stream);
+}
+
 int trie_copy_lists(trie_t h, int64_t *d_offsets, int32_t *d_tokens, cudaStream_t stream) {
     if (!h) return fail(TRIE_EINVAL, "handle is NULL");
     const tmk::DevLists &L = h->lists;
@@ -1309,17 +1350,7 @@ int trie_copy_lists(trie_t h, int64_t *d_offsets, int32_t *d_tokens, cudaStream_
         if (e != cudaSuccess) return fail_cuda(e, "copying the list offsets");
     }
     if (d_tokens && L.n_valid > 0) {
-        // the tokens out of the {token, end node} entries: by a kernel into the
-        // handle's device, by a strided copy into any other memory
-        DeviceGuard g(h->dev.device);
-        cudaPointerAttributes at = {};
-        const bool here = cudaPointerGetAttributes(&at, d_tokens) == cudaSuccess &&
-                          at.type == cudaMemoryTypeDevice && at.device == h->dev.device &&
-                          (reinterpret_cast<uintptr_t>(d_tokens) & 3u) == 0;
-        cudaGetLastError();
-        cudaError_t e = here ? tmk::launch_copy_tokens(L, L.n_valid, d_tokens, num_sms(h->dev.device), stream)
-                             : cudaMemcpy2DAsync(d_tokens, sizeof(int32_t), L.entries, sizeof(int2), sizeof(int32_t),
-                                                 size_t(L.n_valid), cudaMemcpyDeviceToDevice, stream);
+        const cudaError_t e = copy_tokens(h, d_tokens, stream);
         if (e != cudaSuccess) return fail_cuda(e, "copying the list tokens");
     }
     return TRIE_OK;

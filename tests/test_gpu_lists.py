@@ -303,3 +303,57 @@ def test_copy_lists_into_host_memory(cuda):
                                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     torch.cuda.synchronize()
     assert rc == 0 and torch.equal(host, tok.cpu())
+
+
+def test_copy_lists_into_host_memory_time(cuda):
+    """A large list reaches pinned memory in about the time of one copy of its
+    bytes (a copy of one row of 4 bytes an entry takes 16 times as long), and
+    inside a captured graph as well."""
+    import ctypes
+
+    import torch
+    sets = [W.tool_names(s, 1000, 60) for s in range(40)]
+    sb, so = W.pack([x for s in sets for x in s])
+    si = np.cumsum([0] + [len(s) for s in sets]).astype(np.int32)
+    spec = W.VocabSpec(V=32000, max_len=16, substr_frac=0.3, run_frac=0.0, run_len=(2, 4), upper=False, mixed=False)
+    vb, vo = W.byte_vocab(1, spec, substr_src=W.tool_stems(1, 200))
+    h = T.trie_build_many(sb, so, si)
+    n = T.trie_compile_lists(h, vb, vo, spec.V)
+    assert n > 1_000_000
+    _, tok = T.trie_copy_lists(h)
+    host = torch.empty(n, dtype=torch.int32, pin_memory=True)
+
+    def copy(stream):
+        assert h._lib.trie_copy_lists(h.handle, None, ctypes.c_void_p(host.data_ptr()),
+                                      ctypes.c_void_p(stream.cuda_stream)) == 0
+
+    def best(fn):
+        t = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            fn()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+    plain = best(lambda: host.copy_(tok, non_blocking=True))
+    host.fill_(-5)
+    lists = best(lambda: copy(torch.cuda.current_stream()))
+    assert torch.equal(host, tok.cpu())
+    assert lists < 5 * plain, (lists, plain)
+    pageable = np.full(n + 1, -5, np.int32)  # read and written through the host's page tables
+    for off in (0, 1):
+        assert h._lib.trie_copy_lists(h.handle, None, ctypes.c_void_p(pageable.ctypes.data + 4 * off),
+                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        torch.cuda.synchronize()
+        assert np.array_equal(pageable[off:off + n], tok.cpu().numpy())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        copy(torch.cuda.current_stream())
+    for _ in range(2):
+        host.fill_(-5)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(host, tok.cpu())
+    h.destroy()
