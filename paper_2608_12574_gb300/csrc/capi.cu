@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/triemask.h"
+#include "spare_blocks.h"
 #include "tm_internal.h"
 
 namespace {
@@ -992,64 +993,40 @@ int trie_apply_mask(trie_t h, void *d_logits, int dtype, const int32_t *d_states
     return TRIE_OK;
 }
 
-// Blocks of released valid lists kept for the next handles' lists: a fresh
-// block from the pool cost 0.3-0.4 ms of host time for the 4.8 M-node forest
-// (381 MB), more than the list compile's kernels. A block is reused once the
-// event recorded at its release (if any) has completed; at most
-// kSpareListBlocks are kept per device, the largest, the rest go back to the
-// pool.
-constexpr size_t kSpareListBlocks = 2;
-struct SpareBlock {
-    int dev;
-    void *p;
-    size_t bytes;
-    cudaEvent_t ready;  // null: free for use at once
-};
+// Blocks of released valid lists kept for the next handles' lists (which ones:
+// spare_blocks.h): a fresh block from the pool cost 0.3-0.4 ms of host time for
+// the 4.8 M-node forest (381 MB), more than the list compile's kernels. The
+// others go back to the pool.
 static std::mutex g_spare_mu;
-static std::vector<SpareBlock> &g_spare = *new std::vector<SpareBlock>();
+static tmk::SpareBlocks &g_spare = *new tmk::SpareBlocks();
 
-static void *take_spare_block(int dev, size_t bytes) {
+static bool spare_done(void *ready) { return event_done(static_cast<cudaEvent_t>(ready)); }
+
+// *bytes becomes the block's size.
+static void *take_spare_block(int dev, size_t *bytes) {
     std::lock_guard<std::mutex> lk(g_spare_mu);
-    for (size_t i = 0; i < g_spare.size(); i++) {
-        SpareBlock &b = g_spare[i];
-        if (b.dev != dev || b.bytes < bytes || b.bytes > 2 * bytes) continue;
-        if (b.ready) {
-            if (!event_done(b.ready)) continue;
-            cudaEventDestroy(b.ready);
-        }
-        void *p = b.p;
-        g_spare.erase(g_spare.begin() + long(i));
-        return p;
-    }
-    return nullptr;
+    const tmk::SpareBlock b = g_spare.take(dev, *bytes, spare_done);
+    if (!b.p) return nullptr;
+    if (b.ready) cudaEventDestroy(static_cast<cudaEvent_t>(b.ready));
+    *bytes = b.bytes;
+    return b.p;
 }
 
 // Takes a block of `bytes` on device dev (current) whose last use is queued
-// before `ready` (null: none pending). When the cache is full this block takes
-// the place of the smallest smaller one whose last use is over, if there is
-// one, and the other is freed in stream order on `stream`. (Keeping whichever
-// blocks came first, batches of alternating sizes never found one for the
-// largest: 256-request batches of three sizes in turn took 1,067 us each, 903
-// us so.)
+// before `ready` (null: none pending). What is not kept is freed in stream
+// order on `stream`.
 static void give_spare_block(int dev, void *p, size_t bytes, cudaEvent_t ready, cudaStream_t stream) {
-    SpareBlock out{dev, p, bytes, ready};
+    tmk::SpareBlock out;
+    out.dev = dev;
+    out.p = p;
+    out.bytes = bytes;
+    out.ready = ready;
     {
         std::lock_guard<std::mutex> lk(g_spare_mu);
-        size_t held = 0;
-        SpareBlock *least = nullptr;
-        for (SpareBlock &b : g_spare) {
-            if (b.dev != dev) continue;
-            held++;
-            if (b.bytes >= (least ? least->bytes : bytes)) continue;
-            if (!b.ready || event_done(b.ready)) least = &b;
-        }
-        if (held < kSpareListBlocks) {
-            g_spare.push_back(out);
-            return;
-        }
-        if (least) std::swap(*least, out);
+        out = g_spare.give(out, spare_done);
     }
-    if (out.ready) cudaEventDestroy(out.ready);
+    if (!out.p) return;
+    if (out.ready) cudaEventDestroy(static_cast<cudaEvent_t>(out.ready));
     cudaFreeAsync(out.p, stream);
     cudaGetLastError();
 }
@@ -1177,7 +1154,8 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
         const size_t o_tile = lay.add(sizeof(int64_t) * (size_t(n) / 4096 + 2));
         const size_t o_tot = lay.add(sizeof(int64_t));
         const size_t o_tok = by_bound ? lay.add(sizeof(int2) * size_t(std::max<int64_t>(bound, 1))) : 0;
-        void *base = take_spare_block(dev, lay.total);
+        size_t block_bytes = lay.total;
+        void *base = take_spare_block(dev, &block_bytes);
         if (!base && (rc = pool_alloc(dev, lay.total, stream, &base, "the valid lists")) != TRIE_OK) return rc;
         cudaEvent_t done = nullptr;
         cudaError_t e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
@@ -1187,7 +1165,7 @@ static int compile_lists(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, in
         }
         char *b = static_cast<char *>(base);
         L.base = base;
-        L.base_bytes = lay.total;
+        L.base_bytes = block_bytes;
         L.done = done;
         L.count = reinterpret_cast<int32_t *>(b + o_cnt);
         L.off = reinterpret_cast<int64_t *>(b + o_off);
