@@ -339,8 +339,8 @@ int trie_apply_lists(trie_t h, void *d_logits, int dtype, const int32_t *d_state
  *
  * Set-up (host-synchronous; synchronises the device). Allocates, on the
  * current device, (rounded-up cache_rows + max_batch) rows of ceil(V/32)
- * uint32 words plus 52 bytes per trie node (133 for a forest without a dense
- * compile) and 36 per batch row; replaces the cache of an earlier
+ * uint32 words plus 40 bytes per trie node (121 for a forest without a dense
+ * compile; 12 more until it returns) and 36 per batch row; replaces the cache of an earlier
  * trie_lazy_init on the handle (starting empty).
  *   vocab_bytes, vocab_offsets, V  as trie_compile_masks, 2 <= V <= 524,288
  *   cache_rows  rows kept between calls, 0 <= cache_rows <= 2^30 (rounded up

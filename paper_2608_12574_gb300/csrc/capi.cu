@@ -1398,13 +1398,18 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     const size_t o_ctrl = lay.add(sizeof(tmk::LazyCtrl));
     const size_t o_slot = lay.add(sizeof(int32_t) * mb);
     const size_t o_task = lay.add(sizeof(tmk::LazyTask) * (mb + size_t(tmk::kLazySplitRows) * tmk::kLazyMaxParts));
-    const size_t o_pnode = lay.add(sizeof(int32_t) * n);
-    const size_t o_pdep = lay.add(sizeof(int32_t) * n);
-    const size_t o_psize = lay.add(sizeof(int32_t) * n);
     const size_t o_place = lay.add(sizeof(int2) * n);
     const size_t o_pre = lay.add(sizeof(tmk::LazyNode) * n);
-    void *base = nullptr;
+    Layout pre;  // the trie's pre-order, of which the records are made: for the set-up only
+    const size_t o_pnode = pre.add(sizeof(int32_t) * n);
+    const size_t o_pdep = pre.add(sizeof(int32_t) * n);
+    const size_t o_psize = pre.add(sizeof(int32_t) * n);
+    void *base = nullptr, *tmp = nullptr;
     if ((rc = pool_alloc(dev, lay.total, 0, &base, "the lazy rows")) != TRIE_OK) return rc;
+    if ((rc = pool_alloc(dev, pre.total, 0, &tmp, "the lazy rows' set-up")) != TRIE_OK) {
+        pool_free(base);
+        return rc;
+    }
     char *b = static_cast<char *>(base);
     L.device = dev;
     L.base = base;
@@ -1418,27 +1423,28 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     L.ctrl = reinterpret_cast<tmk::LazyCtrl *>(b + o_ctrl);
     L.slot_of = reinterpret_cast<int32_t *>(b + o_slot);
     L.task = reinterpret_cast<tmk::LazyTask *>(b + o_task);
-    L.pre_node = reinterpret_cast<int32_t *>(b + o_pnode);
-    L.pre_depth = reinterpret_cast<int32_t *>(b + o_pdep);
-    L.pre_size = reinterpret_cast<int32_t *>(b + o_psize);
     L.place = reinterpret_cast<int2 *>(b + o_place);
     L.pre = reinterpret_cast<tmk::LazyNode *>(b + o_pre);
+    L.pre_node = reinterpret_cast<int32_t *>(static_cast<char *>(tmp) + o_pnode);
+    L.pre_depth = reinterpret_cast<int32_t *>(static_cast<char *>(tmp) + o_pdep);
+    L.pre_size = reinterpret_cast<int32_t *>(static_cast<char *>(tmp) + o_psize);
     const tmk::LazyCtrl ctrl0 = {1u, 0, 0, 0, 0ull, 0ull};
     const tmk::HostTrie &t = h->host;
     if ((e = cudaMemset(L.tag, 0xFF, sizeof(int32_t) * size_t(C))) != cudaSuccess ||
         (e = cudaMemset(L.stamp, 0, sizeof(uint32_t) * size_t(C))) != cudaSuccess ||
         (e = cudaMemcpy(L.ctrl, &ctrl0, sizeof(ctrl0), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(L.pre_node, t.pre_node.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) !=
-            cudaSuccess ||
-        (e = cudaMemcpy(L.pre_depth, t.pre_depth.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) !=
-            cudaSuccess ||
-        (e = cudaMemcpy(L.pre_size, t.pre_size.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) !=
-            cudaSuccess ||
-        (e = tmk::launch_lazy_tables(h->dev, L, h->host.n, 0)) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess) {
+        (e = cudaMemcpy(L.pre_node, t.pre_node.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(L.pre_depth, t.pre_depth.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(L.pre_size, t.pre_size.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = tmk::launch_lazy_tables(h->dev, L, h->host.n, 0)) != cudaSuccess ||
+        (e = cudaDeviceSynchronize()) != cudaSuccess) {
+        pool_free(tmp);
         pool_free(base);
         L = tmk::DevLazy();
         return fail_cuda(e, "lazy-row set-up");
     }
+    L.pre_node = L.pre_depth = L.pre_size = nullptr;
+    cudaFreeAsync(tmp, 0);  // its only use is over
     L.vocab = voc;
     return TRIE_OK;
 }

@@ -354,7 +354,9 @@ struct DevLazy {
     LazyCtrl *ctrl = nullptr;
     int32_t *slot_of = nullptr;     // [max_batch] row of each batch row, < 0: {EOS}
     LazyTask *task = nullptr;       // [max_batch + kLazySplitRows * kLazyMaxParts]
-    int32_t *pre_node = nullptr;    // [n] pre-order tables of the trie (HostTrie)
+    // the trie's pre-order tables (HostTrie's), of which place and pre are made:
+    // during the set-up only
+    int32_t *pre_node = nullptr;    // [n]
     int32_t *pre_depth = nullptr;   // [n]
     int32_t *pre_size = nullptr;    // [n]
     int2 *place = nullptr;          // [n] pre-order position and subtree size of each node
