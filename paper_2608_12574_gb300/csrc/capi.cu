@@ -825,9 +825,12 @@ static unsigned long long *ensure_seg(trie_t h, int dev, cudaStream_t stream, in
 }
 
 // Tries of up to so many nodes get the arrays of their first dense compile in
-// one block, larger ones the hit buffer and the summary apart: a new schema of
-// 11,500 nodes takes 190 us so and 198 us apart, once; at 23,090 nodes every
-// compile that follows, HBM-write bound, takes 67.2 us so and 66.6 us apart.
+// one block, larger ones the hit buffer and the summary apart. One block saves
+// a new schema 4-9 us once, at every size measured (2,400 to 43,000 nodes). Warm
+// compiles take the same either way at all of them; with other handles'
+// compiles in between, one block takes 67.6 us and apart 67.4 us at 23,090
+// nodes, 504 and 501.5 us at 290,000, for reasons not found. So one block is for
+// tries that are small enough to be compiled once or a few times.
 constexpr int32_t kOneBlockNodes = 16384;
 
 // The mask compile with the vocabulary resolved (from the cache, or a vocabulary handle).
