@@ -220,11 +220,9 @@ __device__ __forceinline__ uint32_t byte_at(const uint32_t (&w)[4], int32_t i) {
 // Whether the token bytes t (zero-padded to 16), k <= 16 of them, are the last
 // k labels of a window (byte i = the label i levels up): token byte j must
 // equal label k - 1 - j, so the token's 16 bytes are reversed and shifted down
-// by 16 - k, which brings byte k - 1 down to byte 0. (Byte by byte, each a
-// select from four registers on either side, the comparison was a good part of
-// the searches' instructions: 8 lazy steps at K = 10,000, B = 256, 217.0 us,
-// 207.6 us so; the compile kernels, whose search runs beside the fill,
-// 505.1 us to 501.3 us at K = 74,719.)
+// by 16 - k, which brings byte k - 1 down to byte 0. Byte by byte, each a select
+// from four registers on either side, the comparison is a good part of the lazy
+// rows' instructions (8 steps at K = 10,000, B = 256: 217.0 us, 207.6 us so).
 __device__ __forceinline__ bool spells_window(const uint32_t (&lab)[4], const uint4 t, int32_t k) {
     const uint64_t win_lo = lab[0] | (uint64_t(lab[1]) << 32), win_hi = lab[2] | (uint64_t(lab[3]) << 32);
     const uint64_t r_lo = __byte_perm(t.w, 0, 0x0123) | (uint64_t(__byte_perm(t.z, 0, 0x0123)) << 32);
@@ -239,11 +237,12 @@ __device__ __forceinline__ bool spells_window(const uint32_t (&lab)[4], const ui
 }
 
 // The same byte by byte, for the quad probe (four lanes a node, 4 lengths a
-// lane), which outlasts the fill beside it: alone, with its tables in L2, the
-// compile of K = 1,000, V = 128,000 takes 33.4 us so and 32.9 us with
-// spells_window, but followed by the 128 decode steps of B = 64 that leave its
-// tables to DRAM, 522 us and 533 us. The other probes are no slower with
-// spells_window there (K = 74,719 with 16 steps 1.107 ms so, 1.101 ms).
+// lane): with spells_window that kernel needs 138 registers, with this 119, which
+// is four CTAs an SM instead of three beside the fill that it outlasts. Alone,
+// with its tables in L2, the compile of K = 1,000, V = 128,000 takes 33.4 us so
+// and 32.9 us with spells_window; followed by the 128 decode steps of B = 64 that
+// leave its tables to DRAM, 522 us and 533 us. The other probes are no slower
+// with spells_window.
 __device__ __forceinline__ bool spells_window_bytes(const uint32_t (&lab)[4], const uint4 t, int32_t k) {
     const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
     bool eq = true;
@@ -1011,12 +1010,10 @@ struct RowCut {
 // TMA bulk copy of the -inf tile; otherwise the lanes write 16-byte chunks,
 // reading the logits only in chunks that hold an allowed token. A lane reads up
 // to 4 chunks before its first store, so that it waits for DRAM once (bf16, 4
-// chunks a lane) or twice (fp32, 8). One after the other, 8 steps of K = 10,000,
-// V = 152,064, B = 256 in bf16 took 116.5 us, 109.7 us so. All 8 of an fp32 lane
-// at a time take 54 registers in the fused kernel, 4 resident CTAs an SM
-// instead of 6: B = 256, V = 262,144 37.3 us a launch, 36.8 us so, and the compile
-// of K = 74,719 with 16 steps 1.123 ms, 1.098 ms so (rows that do not start on a
-// 16-byte boundary, V = 152,063, 24.1 us a launch and 24.5 us so).
+// chunks a lane) or twice (fp32, 8): 8 steps of K = 10,000, V = 152,064, B = 256
+// in bf16 take 109.7 us so and 116.5 us one chunk after the other. All 8 of an
+// fp32 lane at a time take 54 registers in the fused kernel, 4 resident CTAs an
+// SM instead of 6 (B = 256, V = 262,144 37.3 us a launch, 36.8 us so).
 // Stores are evict-first: the logits stream must not flush the trie tables.
 template <int kElt>
 __device__ __forceinline__ void write_segment(const RowCut<kElt> &row, int32_t seg, uint32_t word,
@@ -1366,14 +1363,12 @@ __global__ void k_rt_insert(const int32_t *__restrict__ parent, const uint8_t *_
 // the reversed trie's root for byte c. The climb reads each level's parent
 // and label itself, one level ahead of the edge it looks up: neighbouring
 // nodes' ancestors are neighbours, so these loads fall together and come from
-// L1 and L2, where reading each entry's row from the 64-byte ancestor rows of
-// the dense compile's tables was 305 MB of DRAM reads a walk on the 4.77 M-node
-// forest (count walk 132 us, 98 us so; write walk 177 and 135 us; and the
-// forest needs no such tables). Bound by the L1's look-ups of the random edge
-// slots (two, three or four nodes a lane, their loads side by side: 8, 117 and
-// 112 us more for both walks together). Called by whole warps, whose lanes stay
-// together until the longest walk ends: with a return at each lane's own end
-// the lanes ran on one by one (326 and 520 us).
+// L1 and L2 (98 us the count walk and 135 us the write walk on the 4.77 M-node
+// forest; 132 and 177 us from the dense compile's 64-byte ancestor rows, 305 MB
+// of DRAM reads a walk). Bound by the L1's look-ups of the random edge slots, so
+// that more nodes a lane, their loads side by side, gain nothing. Called by
+// whole warps, whose lanes stay together until the longest walk ends: with a
+// return at each lane's own end the lanes run on one by one (326 and 520 us).
 template <typename Tok>
 __device__ __forceinline__ void walk_node(const WalkArgs &a, const int2 *root, int32_t m, Tok tok) {
     int32_t p = -1, x = -1, t = -1;  // (x, t): the edge taken by the label below p
@@ -1570,9 +1565,8 @@ __device__ __forceinline__ int32_t lazy_set(int32_t s, int32_t n_sets) {
 // and for a missing node its place and stamps (both at once) and the claim; a
 // thread keeps its batch rows' results in registers and the missing nodes stay
 // in shared memory, so nothing is passed on through L2 between the phases
-// (K = 10,000, B = 256, no cache: 6.7-7.1 us of a step from the apply before
-// to its end, 4.6-6.4 us so; without a cache, tasks added by whoever enters a
-// node in the first phase gained nothing).
+// (K = 10,000, B = 256, no cache: 4.6-6.4 us of a step from the apply before
+// to its end, 6.7-7.1 us through L2).
 constexpr int kResolvePer = kLazyMaxBatch / kResolveThreads;  // batch rows per thread
 
 template <bool kAdvance>
@@ -1756,14 +1750,13 @@ __device__ __forceinline__ uint64_t hash_pow(uint32_t j) {
 }
 
 // A task's row is a chain of loads: task, records, slot pair, payload, token
-// bytes (12 us of a step at K = 10,000, B = 256 with the node's place looked up
-// again and the token's id, length and bytes one after the other, 7.8-9.4 us
-// so). The moves it found are kept until the row is stored: inserted as they
-// are found, each one's compare-and-swap in the transition table held up the
-// row. (Moves beyond the list are inserted at once. A look at the slot before
-// the compare-and-swap gained nothing.) The first task is read beside the
-// tasks' count, whole rows are stored 16 bytes at a time, and the powers of the
-// hash's base come from shared memory: 24.2 us a step before these, 23.4 us so.
+// bytes (7.8-9.4 us of a step at K = 10,000, B = 256; 12 us with the token's id,
+// length and bytes one after the other). The moves it found are kept until the
+// row is stored (beyond the list they are inserted at once): each one's
+// compare-and-swap in the transition table would hold up the row. The first task
+// is read beside the tasks' count, whole rows are stored 16 bytes at a time, and
+// the powers of the hash's base come from shared memory (23.4 us a step, 24.2
+// without these three).
 constexpr int kLazyMoves = 256;
 constexpr int kLazyPows = 32;  // powers of the hash's base kept in shared memory
 

@@ -99,7 +99,8 @@ __device__ __forceinline__ void trie_links(const int32_t *__restrict__ parent, c
     }
 }
 
-// Per-node tables of the probe and of the list walk (one thread per node,
+// Per-node tables of the dense compile's probe and of the lazy rows' set-up
+// (which keeps the label windows in its records; one thread per node,
 // climbing at most 16 parents): the last 16 edge labels into m (byte i = the
 // label i levels up, 0 past the root), min(depth, 16), and the 16 nearest
 // ancestors (-1 past the root), stored as four 16-byte rows. Siblings and

@@ -257,7 +257,7 @@ struct DevTrie {
     ulonglong2 *trans = nullptr;     // transition table {(row << 32 | token) + 1, end node}
     uint32_t trans_mask = 0;         // slots - 1
     bool trans_clean = false;        // the table was cleared at the upload and not used since
-    // Segment summary of the dense mask (own allocation): per row, words of 32
+    // Segment summary of the dense mask: per row, words of 32
     // segment bits (1,024 tokens each) tagged in their high half with the
     // epoch of the compile that set them; a word with another tag than the
     // device's current epoch (*seg_epoch, written by each compile's probe)
@@ -299,11 +299,10 @@ constexpr int32_t kLazyMaxCacheRows = int32_t(1) << 30;  // cache rows + call ro
 constexpr int64_t kLazyMaxWords = 16384;  // row built in shared memory (64 KB): V <= 524,288
 // A missing row whose subtree has more than kLazyPartNodes nodes is computed
 // in parts by several CTAs (at most kLazyMaxParts per row), for at most
-// kLazySplitRows rows per call: a subtree left whole is one CTA's, and a step
-// of K = 74,719, V = 262,144, B = 256 without a cache, whose 26 letters hold
-// 4,300 nodes each, took 70.5 us with 16 rows, 67.4 with 32, 65.1 with 64, 65.6
-// with 128 (parts of 512, 1,536 and 2,048 nodes with 64 rows: 70.5, 66.3 and
-// 66.4 us; K = 10,000 24.3 us with 1,024, 25.1-25.5 us with the others).
+// kLazySplitRows rows per call: a subtree left whole is one CTA's. A step of
+// K = 74,719, V = 262,144, B = 256 without a cache, whose 26 letters hold 4,300
+// nodes each, takes 70.5 us with 16 rows, 65.1 us with 64 and 65.6 us with 128;
+// parts of 512 or 2,048 nodes take 70.5 and 66.4 us.
 constexpr int32_t kLazyPartNodes = 1024;
 constexpr int32_t kLazyMaxParts = 64;
 constexpr int32_t kLazySplitRows = 64;
