@@ -430,12 +430,14 @@ int ensure_device_trie(trie_t h, int dev, cudaStream_t stream, int32_t dense_wor
 
 // The transition table holds transitions of one vocabulary: when a compile
 // uses another, clear it and let this compile's probe refill it; when it
-// holds only the entries lazy rows added, let the compile complete it.
+// holds only the entries lazy rows added, let the compile complete it. A clear
+// and a fill that were captured may never run, so the next call outside the
+// graph makes its own.
 int prepare_trans(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, int sms, cudaStream_t stream, bool *fill) {
     std::lock_guard<std::mutex> lk(h->mu);
     *fill = false;
     if (!h->dev.trans) return TRIE_OK;
-    if (h->trans_vocab == voc) {
+    if (h->trans_vocab == voc && !h->dev.trans_captured) {
         *fill = !h->trans_complete;
         return TRIE_OK;
     }
@@ -446,6 +448,7 @@ int prepare_trans(trie_t h, const std::shared_ptr<tmk::DevVocab> &voc, int sms, 
         if (e != cudaSuccess) return fail_cuda(e, "transition table clear");
     }
     h->dev.trans_clean = false;
+    h->dev.trans_captured = is_capturing(stream);
     *fill = true;
     return TRIE_OK;
 }
@@ -1379,12 +1382,13 @@ int trie_lazy_init(trie_t h, const uint8_t *vocab_bytes, const int64_t *vocab_of
     if ((rc = ensure_tables(h, dev, 0)) != TRIE_OK) return rc;
     {  // the transition table takes the moves the lazy rows find for this vocabulary
         std::lock_guard<std::mutex> lk(h->mu);
-        if (h->dev.trans && h->trans_vocab != voc) {
+        if (h->dev.trans && (h->trans_vocab != voc || h->dev.trans_captured)) {
             h->trans_vocab.reset();
             h->trans_complete = false;
             if (!h->dev.trans_clean && (e = tmk::launch_trans_clear(h->dev, num_sms(dev), 0)) != cudaSuccess)
                 return fail_cuda(e, "transition table clear");
             h->dev.trans_clean = false;
+            h->dev.trans_captured = false;
             h->trans_vocab = voc;
         }
     }

@@ -257,6 +257,7 @@ struct DevTrie {
     ulonglong2 *trans = nullptr;     // transition table {(row << 32 | token) + 1, end node}
     uint32_t trans_mask = 0;         // slots - 1
     bool trans_clean = false;        // the table was cleared at the upload and not used since
+    bool trans_captured = false;     // its last clear and fill were captured (and may not have run)
     // Segment summary of the dense mask: per row, words of 32
     // segment bits (1,024 tokens each) tagged in their high half with the
     // epoch of the compile that set them; a word with another tag than the

@@ -109,3 +109,50 @@ def test_first_compile_captured(build, uploaded):
         assert np.array_equal(first.cpu().numpy().view(np.uint32), want)
     del g
     h.destroy()
+
+
+@pytest.mark.parametrize("then", ["masks", "lazy"])
+def test_moves_after_a_captured_compile(then):
+    """A single trie's transition table, whose clear and fill were captured but
+    have not run, in memory where an earlier handle's table lies: the same rows
+    and tokens with the moves of another vocabulary."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    oracle.build()
+    strings, toks = random_case(91)
+    sb, so = W.pack(strings)
+    V = len(toks)
+    other = T.trie_vocab_create(*W.pack(toks[-2::-1] + toks[-1:]), V)  # every token but EOS under another id
+    vb, vo = W.pack(toks)
+    voc = T.trie_vocab_create(vb, vo, V)
+    ot, ov = oracle.Trie(sb, so), oracle.Vocab(vb, vo)
+    n = ot.num_nodes
+    masks = torch.empty((2, n, T.mask_words(V)), dtype=torch.int32, device="cuda")
+    for _ in range(3):  # the pool's next block of this size is one of these
+        old = T.trie_build(sb, so)
+        T.trie_compile_lists_vocab(old, other)
+        T.trie_compile_masks_vocab(old, other, masks[0])
+        old.destroy()
+    h = T.trie_build(sb, so)
+    T.trie_compile_lists_vocab(h, voc)  # the upload, as the old handle's
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        T.trie_compile_masks_vocab(h, voc, masks[1])
+    s0 = np.repeat(np.arange(n, dtype=np.int32), V)
+    t0 = np.tile(np.arange(V, dtype=np.int32), n)
+    want, _ = oracle.advance(ot, ov, s0, t0)
+    states, tokens = torch.as_tensor(s0, device="cuda"), torch.as_tensor(t0, device="cuda")
+    for k in range(2):
+        if k == 1:
+            g.replay()
+        elif then == "masks":
+            T.trie_compile_masks_vocab(h, voc, masks[0])
+        else:
+            T.trie_lazy_init(h, vb, vo, V, cache_rows=0, max_batch=8)
+        got = states.clone()
+        T.trie_advance(h, got, tokens)
+        assert np.array_equal(got.cpu().numpy(), want)
+    del g
+    h.destroy()
