@@ -696,8 +696,9 @@ int trie_build_many_device(const uint8_t *bytes, const int64_t *offsets, const i
             delete h;
             return fail(TRIE_EINVAL, "offsets must be non-negative and non-decreasing");
         }
-        // long strings (a long level loop) or many sets with deep strings
-        // (the per-(set, depth) tables): the host builder
+        // long strings (a long level loop; a length has 16 bits in the sort) or
+        // many sets with deep strings (the level path's per-(set, depth)
+        // tables): the host builder
         if (e == cudaSuccess &&
             (max_len > tmk::kDeviceBuildMaxDepth || int64_t(M) * (max_len + 1) > tmk::kDeviceBuildMaxGroups)) {
             delete h;

@@ -270,7 +270,7 @@ def trie_build_many(set_bytes, set_offsets, set_index) -> Trie:
 
 
 def trie_build_many_device(set_bytes, set_offsets, set_index, stream=None) -> Trie:
-    """trie_build_many with the level loop on the current CUDA device (same node layout)."""
+    """trie_build_many on the current CUDA device (same node layout)."""
     import torch
     lib = load_library()
     b = _host(set_bytes, np.uint8)

@@ -250,7 +250,7 @@ def test_device_forest_single_set_mask_equals_oracle(cuda):
 
 
 def test_device_forest_long_strings_use_the_host_builder(cuda):
-    """Strings longer than the level loop's limit (1,024 bytes) go to the host
+    """Strings longer than the device build's limit (1,024 bytes) go to the host
     builder; the result is the same forest."""
     rng = np.random.default_rng(11)
     long = bytes(rng.integers(0, 3, 1500, dtype=np.uint8))

@@ -6,6 +6,7 @@ rows are evicted and recomputed within one decode loop.
 """
 from __future__ import annotations
 
+import itertools
 import os
 
 import numpy as np
@@ -214,7 +215,7 @@ def test_lazy_decode_equals_dense(cuda, cfg, cache):
 @pytest.mark.parametrize("V", [33, 1001, 4096])
 def test_lazy_apply_random_bits(cuda, dtype, V):
     """Allowed logits keep their exact bits (NaN payloads, -0.0); the rest
-    become -inf; V = 33 and 1001 take the one-thread-per-logit path."""
+    become -inf; with V = 33 and 1001 rows start off the 16-byte boundaries."""
     import torch
     r = np.random.default_rng(V + 7)
     strings = [bytes(r.integers(97, 100, r.integers(1, 6))) for _ in range(30)]
@@ -377,3 +378,67 @@ def test_lazy_large_batch_small_cache(cuda):
         total += int((states >= 0).sum())
     hits, misses = T.trie_lazy_stats(h)
     assert hits + misses == total and hits > 0
+
+
+def _prefix_closed(letters: bytes, d: int) -> list[bytes]:
+    """The first d strings over the letters, by length (every prefix of one is one)."""
+    out, level = [], [b""]
+    while len(out) < d:
+        level = [x + bytes([c]) for x in level for c in letters]
+        out += level
+    return out[:d]
+
+
+@pytest.mark.parametrize("pad", [0, 1, 2, 3])
+def test_lazy_rows_by_subtree_size(cuda, pad):
+    """Subtrees of a CTA's threads' one descendant each and of one more, of one
+    part's nodes and of one more, and of several parts, whose rows hold more
+    moves than a task keeps (256); rows of every number of words modulo 4."""
+    import torch
+    sizes = [1, 255, 256, 257, 1024, 1025, 2049, 3000]
+    strings = [bytes([65 + i]) + x for i, d in enumerate(sizes) for x in _prefix_closed(b"abc", d)]
+    toks = _prefix_closed(b"abc", 1092) + [bytes([65 + i]) for i in range(len(sizes))]
+    toks += [b"Z%d" % i for i in range(1119 + 32 * pad - len(toks))] + [b""]  # V = 35, 36, 37, 38 words
+    sb, so = W.pack(strings)
+    vb, vo = W.pack(toks)
+    V = len(toks)
+    assert (V + 31) // 32 % 4 == (3 + pad) % 4
+    h = T.trie_build(sb, so)
+    ot, ov = oracle.Trie(sb, so), oracle.Vocab(vb, vo)
+    assert ot.num_nodes == 1 + len(sizes) + sum(sizes)
+    T.trie_lazy_init(h, vb, vo, V, cache_rows=0, max_batch=64)
+    states = np.arange(1 + len(sizes), dtype=np.int32)  # the root and the sizes' nodes
+    want = _want_rows(ot, ov, states, V)
+    assert np.array_equal(_rows(cuda, h, states, V), want)
+    for s in states:
+        assert np.array_equal(_rows(cuda, h, [s], V)[0], want[s]), int(s)
+    # the moves that the rows' searches recorded
+    s0, t0 = np.repeat(states, V), np.tile(np.arange(V, dtype=np.int32), len(states))
+    got = torch.as_tensor(s0, device=cuda)
+    new = torch.empty_like(got)
+    x = torch.zeros((64, V), device=cuda)
+    end, _ = oracle.advance(ot, ov, s0, t0)
+    for a in range(0, len(s0), 64):
+        n = min(64, len(s0) - a)
+        T.trie_lazy_advance_apply(h, got[a:a + n], torch.as_tensor(t0[a:a + n], device=cuda), new[a:a + n], x[:n])
+    assert np.array_equal(new.cpu().numpy(), end)
+
+
+@pytest.mark.parametrize("cache", [0, 1024])
+def test_lazy_more_large_subtrees_than_are_split(cuda, cache):
+    """73 nodes of more than 1,024 descendants in one call: 64 of their rows are
+    built in parts, the others whole, each with thousands of tokens."""
+    letters = b"abcdefgh"
+    leaves = [bytes(x) for x in itertools.product(letters, repeat=6)]
+    toks = _prefix_closed(letters, 8 + 64 + 512 + 4096) + [b""]
+    sb, so = W.pack(leaves)
+    vb, vo = W.pack(toks)
+    V = len(toks)
+    h = T.trie_build(sb, so)
+    ot, ov = oracle.Trie(sb, so), oracle.Vocab(vb, vo)
+    states = np.arange(73, dtype=np.int32)  # depths 0, 1 and 2
+    T.trie_lazy_init(h, vb, vo, V, cache_rows=cache, max_batch=128)
+    want = _want_rows(ot, ov, states, V)
+    order = np.random.default_rng(1).permutation(73).astype(np.int32)
+    for _ in range(2):
+        assert np.array_equal(_rows(cuda, h, order, V), want[order])

@@ -244,8 +244,8 @@ def test_decode_loop_lists_fused(cuda, cfg):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [33, 1001, 8193])
 def test_advance_apply_lists_random(cuda, dtype, V):
-    """Random states (invalid ones included) and tokens, the scalar path for
-    V = 33 / 1001: states against the oracle's advance, logits against its
+    """Random states (invalid ones included) and tokens, rows off the 16-byte
+    boundaries for V = 33 / 1001: states against the oracle's advance, logits against its
     apply by the new states."""
     import torch
     r = np.random.default_rng(V + 3)

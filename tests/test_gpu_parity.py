@@ -265,7 +265,7 @@ def test_advance_long_paths(cuda):
 @pytest.mark.parametrize("V", [2, 33, 1001, 4096, 32000])
 def test_apply_random_bits(cuda, dtype, V):
     """Every bit pattern (NaN payloads, -0.0) of an allowed logit survives; the rest become -inf.
-    V = 33 and 1001 take the unaligned one-thread-per-logit path."""
+    With V = 33 and 1001 rows start off the 16-byte boundaries."""
     import torch
     r = np.random.default_rng(V)
     strings = [bytes(r.integers(97, 100, r.integers(1, 6))) for _ in range(30)]
@@ -287,7 +287,7 @@ def test_apply_random_bits(cuda, dtype, V):
     assert np.array_equal(_bits(x), want)
 
 
-def test_apply_unaligned_base_uses_scalar_path(cuda):
+def test_apply_unaligned_base(cuda):
     import torch
     sb, so = W.pack([b"ab", b"b"])
     toks = [bytes([c]) for c in range(256)] + [b"ab"] * 7 + [b""]
