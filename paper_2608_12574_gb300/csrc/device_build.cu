@@ -549,9 +549,10 @@ __global__ void __launch_bounds__(kSetThreads, 3) k_b_set_sort(const uint8_t *__
     extern __shared__ uint4 dyn[];
     ulonglong2 *key = reinterpret_cast<ulonglong2 *>(dyn);
     uint16_t *len = reinterpret_cast<uint16_t *>(key + 2 * size_t(cap));
-    uint16_t *const pos = len + cap, *const lcp = pos + cap;  // the order, and what each string shares with the one before
-    uint16_t *list = lcp + cap, *buf = list + cap;            // the strings to sort, and the sort's other side
+    uint16_t *pos = len + cap, *const lcp = pos + cap;  // the order, and what each string shares with the one before
+    uint16_t *list = lcp + cap, *buf = list + cap;      // the strings to sort, and the sort's other side
     __shared__ int32_t ws[kSetThreads / 32];
+    __shared__ int2 sums[kSetThreads / 32];
     __shared__ uint8_t edge[kSetThreads + 1];
     pdl_launch_dependents();
     pdl_wait();
@@ -585,9 +586,15 @@ __global__ void __launch_bounds__(kSetThreads, 3) k_b_set_sort(const uint8_t *__
         while (true) {
             if (!in_order) {
                 sort_strings(str, list, buf, listed);
-                for (int32_t k = 0, at = at0; k < r1 - r0; k++)
-                    if ((tied >> k) & 1u) pos[r0 + k] = list[at++];
-                __syncthreads();
+                if (str.base == 0) {  // every string, so the list is the order
+                    uint16_t *const t = pos;
+                    pos = list;
+                    list = t;
+                } else {
+                    for (int32_t k = 0, at = at0; k < r1 - r0; k++)
+                        if ((tied >> k) & 1u) pos[r0 + k] = list[at++];
+                    __syncthreads();
+                }
             }
             for (int32_t k = 0; k < r1 - r0; k++) {
                 if (!((joined >> k) & 1u)) continue;
@@ -635,12 +642,18 @@ __global__ void __launch_bounds__(kSetThreads, 3) k_b_set_sort(const uint8_t *__
             nodes += l - c;
             if (i == 0 || c < l) my_chars += l;  // not a repetition of the string before it
         }
-        int32_t total, total_chars;
-        set_excl_scan(nodes, ws, &total);
-        set_excl_scan(my_chars, ws, &total_chars);
-        if (tid == 0) {
-            count[s] = 1 + total;
-            if (total_chars) atomicAdd(chars, static_cast<unsigned long long>(total_chars));
+        nodes = __reduce_add_sync(0xffffffffu, nodes);
+        my_chars = __reduce_add_sync(0xffffffffu, my_chars);
+        if ((tid & 31) == 0) sums[tid >> 5] = make_int2(nodes, my_chars);
+        __syncthreads();
+        if (tid < 32) {
+            const int2 v = tid < kSetThreads / 32 ? sums[tid] : make_int2(0, 0);
+            nodes = __reduce_add_sync(0xffffffffu, v.x);
+            my_chars = __reduce_add_sync(0xffffffffu, v.y);
+            if (tid == 0) {
+                count[s] = 1 + nodes;
+                if (my_chars) atomicAdd(chars, static_cast<unsigned long long>(my_chars));
+            }
         }
     }
 }
